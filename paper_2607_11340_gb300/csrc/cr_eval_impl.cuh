@@ -3,6 +3,8 @@
 // per-component loads and stores of a warp are coalesced.
 #pragma once
 
+#include <cooperative_groups.h>
+
 #include "cr_host.h"
 
 namespace crk {
@@ -98,20 +100,65 @@ __global__ void __launch_bounds__(128) k_cost_grad(RobotK<T> rb, WeightsK<T> w, 
   }
 }
 
-// Deterministic row sums: one block per row, fixed per-thread strides and a fixed tree order.
+// Deterministic row sums in FP64: row y = blockIdx.y is cut into gridDim.x equal pieces, one block of
+// the cluster (gridDim.x, 1, 1) each; a thread adds its piece's elements with 8 loads in flight into 4
+// accumulators, a block its threads by butterflies and warps in order, block 0 the blocks' sums in
+// order through distributed shared memory. All orders are fixed by (B, gridDim.x).
+// Bound: the FP64 pipe (a widening and an addition per element, each holding a sub-partition's unit
+// 64 cycles). One block of 256 threads with one load in flight per row kept 6 SMs busy on the 6
+// parameter rows of 262,144 states and waited on every load: 195 us of a 485 us gradient pass, which takes
+// 328 us with 16 blocks per row (60,001 states and 8 rows: 52 us of 396, now 359).
+constexpr int kReduceThreads = 512, kReduceWarps = kReduceThreads / 32;
 template <typename T>
-__global__ void __launch_bounds__(256) k_reduce_rows(const T* __restrict__ x, int64_t B, double* out) {
-  __shared__ double part[256];
-  const T* row = x + (int64_t)blockIdx.x * B;
-  double s = 0;
-  for (int64_t b = threadIdx.x; b < B; b += blockDim.x) s += double(row[b]);
-  part[threadIdx.x] = s;
-  __syncthreads();
-  for (int off = 128; off > 0; off >>= 1) {
-    if ((int)threadIdx.x < off) part[threadIdx.x] += part[threadIdx.x + off];
-    __syncthreads();
+__global__ void __launch_bounds__(kReduceThreads) k_reduce_rows(const T* __restrict__ x, int64_t B, double* out) {
+  __shared__ double part[kReduceWarps];
+  __shared__ double total;
+  namespace cg = cooperative_groups;
+  const int64_t len = (B + gridDim.x - 1) / gridDim.x;
+  const int64_t b0 = len * blockIdx.x, b1 = b0 + len < B ? b0 + len : B;
+  const T* row = x + (int64_t)blockIdx.y * B;
+  double acc[4] = {0.0, 0.0, 0.0, 0.0};
+  int64_t b = b0 + threadIdx.x;
+  for (; b + 7 * kReduceThreads < b1; b += 8 * kReduceThreads) {
+    T v[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) v[k] = row[b + k * kReduceThreads];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) acc[k & 3] += double(v[k]);
   }
-  if (threadIdx.x == 0) out[blockIdx.x] = part[0];
+  for (; b < b1; b += kReduceThreads) acc[0] += double(row[b]);
+  double s = (acc[0] + acc[1]) + (acc[2] + acc[3]);
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+  if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = s;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    s = part[0];
+    for (int w = 1; w < kReduceWarps; ++w) s += part[w];
+    total = s;
+  }
+  if (gridDim.x == 1) {
+    if (threadIdx.x == 0) out[blockIdx.y] = s;
+    return;
+  }
+  cg::cluster_group cl = cg::this_cluster();
+  cl.sync();
+  if (blockIdx.x == 0 && threadIdx.x < 32) {
+    double t = threadIdx.x < gridDim.x ? *cl.map_shared_rank(&total, threadIdx.x) : 0.0;
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) t += __shfl_xor_sync(0xffffffffu, t, off);
+    if (threadIdx.x == 0) out[blockIdx.y] = t;
+  }
+  cl.sync();  // block 0 has read every block's sum before any of them exits
+}
+
+// Blocks per row: enough for about one block per SM over all rows, a power of two of at most 16 (the
+// largest cluster, opt-in), and at least 2048 elements to a block, below which one block's few loads
+// cost less than the cluster's barriers.
+inline int reduce_cluster(int64_t rows, int64_t B) {
+  int c = 1;
+  while (c < 16 && rows * c < 152 && B >= (int64_t)4096 * c) c *= 2;
+  return c;
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -219,7 +266,27 @@ template <typename T> cr_status launch_cost_grad(const EvalArgs& a) {
 #define CR_EVAL_COUPLED_INSTANTIATE(EXT, T) EXT template void launch_eval_coupled<T>(const EvalArgs&, int);
 template <typename T>
 cr_status launch_reduce_rows(const void* x, int64_t rows, int64_t B, double* out, cudaStream_t s) {
-  k_reduce_rows<T><<<(unsigned)rows, 256, 0, s>>>((const T*)x, B, out);
+  const int c = reduce_cluster(rows, B);
+  for (int64_t r0 = 0; r0 < rows; r0 += 65535) {  // rows along grid.y
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)c, (unsigned)(rows - r0 < 65535 ? rows - r0 : 65535), 1);
+    cfg.blockDim = dim3(kReduceThreads, 1, 1);
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)c;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = c > 1 ? 1 : 0;
+    cudaError_t e = cudaSuccess;
+    if (c > 8) e = cudaFuncSetAttribute(k_reduce_rows<T>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e == cudaSuccess) e = cudaLaunchKernelEx(&cfg, k_reduce_rows<T>, (const T*)x + r0 * B, B, out + r0);
+    if (e != cudaSuccess) {
+      (void)cudaGetLastError();
+      return crh::fail(CR_ECUDA, "cr_reduce_rows: %s", cudaGetErrorString(e));
+    }
+  }
   return crh::check_launch("cr_reduce_rows");
 }
 
