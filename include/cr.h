@@ -503,12 +503,12 @@ CR_API size_t cr_calibrate_workspace_size(const cr_robot* robot, int64_t K);
 /* LM calibration of theta = (L_1..n, r_c,1..n) from K known displacements U [3n][K] (`dtype`) and
  * measured tip positions P_meas [3][K] (FP64): residual p(u_k; theta) - p_k. theta (device, FP64,
  * [2n]) holds the initial guess and receives the estimate; F_out (device, [1]) the final cost;
- * hist (device, nullable, [iters][2n]) the iterates. Same LM rule as cr_lm_step; J^T J and J^T r
- * reduced in FP64 in a fixed order (per block of 128 poses, then over the blocks in order),
- * Cholesky in FP64. Per iteration one many-block launch forms the partial sums and one single-block
- * launch solves, evaluates the trial cost and applies the rule. `workspace` (device, 8-byte
- * aligned, at least cr_calibrate_workspace_size bytes, caller-owned) holds the damping state and
- * the partial sums; it is overwritten. */
+ * hist (device, nullable, [iters][2n]) the iterates. Same LM rule as cr_lm_step; J^T J, J^T r and F
+ * reduced in FP64 in a fixed order, the damped system solved in FP64 by the symmetric sweep (the pivots of
+ * its LDL^T factorisation). One launch per iteration: it applies the rule to the last trial point, solves
+ * for the next and evaluates there. `workspace` (device, 8-byte aligned, at least
+ * cr_calibrate_workspace_size bytes, caller-owned) holds the LM state and the partial sums; it is
+ * overwritten. */
 CR_API cr_status cr_calibrate(const cr_robot* robot, const void* U, const double* P_meas, int64_t K, double* theta,
                               int32_t iters, double lambda0, double* F_out, double* hist, int32_t dtype,
                               void* workspace, size_t ws_bytes, cr_stream stream);

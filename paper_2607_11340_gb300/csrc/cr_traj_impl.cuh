@@ -425,19 +425,134 @@ __device__ void calib_rows(const RobotK<T>& rb, const T (&u)[3 * N], const doubl
   }
 }
 
-// Multi-block form. Per LM iteration, k_calib_accum (one thread per pose, 128 poses per block) adds
-// each block's contributions to J^T J (packed), J^T r and F = 1/2 sum r^2 in FP64 (warp butterflies,
-// then the four warps in order) into part[block][.]; k_calib_step (one block) adds the partials in
-// block order, factors the damped system in FP64, evaluates the trial cost over all poses and applies
-// the LM rule to theta (in place), lambda and nu (workspace). All sums have a fixed order.
-constexpr int kCalibThreads = 128;
+// FP64 form of calib_rows with what the radius column does not need left out: theta scales with 1 / r_c,
+// so that column is the derivative along the bend's own direction, a turn about the bend's fixed axis
+// w = (-ay, ax, 0) (J_l(w) w = w) and L d(c ax, c ay, s)/dscale = L (ax (c + 2x c'), ay (c + 2x c'), 2x s').
+// The four coefficients are Taylor polynomials up to theta = 3.1417 (seg_coef_poly), the library's sine and
+// cosine beyond. About 600 FP64 instructions a pose and three segments against 1000 through
+// segment_twists; each holds a sub-partition's FP64 unit 64 cycles.
+constexpr double inv_fact(int n) {
+  double f = 1.0;
+  for (int k = 2; k <= n; ++k) f *= double(k);
+  return 1.0 / f;
+}
+// sum_{k < M} (-1)^k c_k z^k with c_k = 1 / (2k + A)! (times k + 1 with LIN), by Horner's rule. 12 terms in
+// y = x / 4 <= 2.468 and 14 in x <= 9.87 leave less than 1e-17 of the leading term.
+template <int M, int A, bool LIN> CR_HD double taylor_alt(double z) {
+  double v = 0.0;
+#pragma unroll
+  for (int k = M - 1; k >= 0; --k) {
+    const double c = (k % 2 ? -1.0 : 1.0) * (LIN ? double(k + 1) : 1.0) * inv_fact(2 * k + A);
+    v = k == M - 1 ? c : fma(v, z, c);
+  }
+  return v;
+}
+CR_HD void seg_coef_poly(double x, double& s, double& c, double& s3, double& cp) {
+  if (x <= double(kPolyMaxX)) {
+    const double y = 0.25 * x;
+    const double sc = taylor_alt<12, 1, false>(y);  // sinc(theta / 2)
+    s = sc * taylor_alt<12, 0, false>(y);
+    c = 0.5 * sc * sc;
+    s3 = taylor_alt<14, 3, false>(x);
+    cp = -taylor_alt<14, 4, true>(x);
+  } else {
+    seg_sc_lib(x, s, c);
+    seg_deriv_lib(x, s, c, s3, cp);
+  }
+}
+template <typename T, int N>
+__device__ void calib_pose(const RobotK<T>& rb, const T (&u)[3 * N], const double* pm, T (&r)[3], T (&J)[3][2 * N]) {
+  calib_rows<T, N>(rb, u, pm, r, J);
+}
+template <int N>
+__device__ void calib_pose_f64(const RobotK<double>& rb, const double (&u)[3 * N], const double* pm, double (&r)[3],
+                               double (&J)[3][2 * N]) {
+  double R[9] = {1.0, 0.0, 0.0, 0.0, 1.0, 0.0, 0.0, 0.0, 1.0}, p[3] = {0.0, 0.0, 0.0};
+  double v[N][3], wv[N][3], pe[N][3];
+#pragma unroll
+  for (int i = 0; i < N; ++i) {
+    double ax, ay, s, c, s3, cp;
+    bend_of(rb.K[i], u[3 * i], u[3 * i + 1], u[3 * i + 2], ax, ay);
+    const double x = ax * ax + ay * ay, L = rb.L[i];
+    seg_coef_poly(x, s, c, s3, cp);
+    const double d[3] = {c * ax, c * ay, s};
+    const double q = L * fma(2.0 * x, cp, c);
+    const double dd[3] = {q * ax, q * ay, L * x * (s3 - c)};  // 2x s' = x (s3 - c)
+    if (i == 0) {  // base frame = identity
+#pragma unroll
+      for (int a = 0; a < 3; ++a) { J[a][i] = d[a]; v[i][a] = dd[a]; }
+      wv[i][0] = -ay; wv[i][1] = ax; wv[i][2] = 0.0;
+    } else {
+      double t[3];
+      matvec(R, d, t);
+#pragma unroll
+      for (int a = 0; a < 3; ++a) J[a][i] = t[a];
+      matvec(R, dd, v[i]);
+#pragma unroll
+      for (int a = 0; a < 3; ++a) wv[i][a] = R[3 * a + 1] * ax - R[3 * a] * ay;
+    }
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      p[a] = fma(L, J[a][i], p[a]);
+      pe[i][a] = p[a];
+    }
+    if (i + 1 < N) {
+      double Ri[9], di[3];
+      seg_transform(ax, ay, x, s, c, L, Ri, di);
+      if (i == 0) {
+#pragma unroll
+        for (int a = 0; a < 9; ++a) R[a] = Ri[a];
+      } else {
+        double Rn[9];
+#pragma unroll
+        for (int a = 0; a < 3; ++a)
+#pragma unroll
+          for (int b = 0; b < 3; ++b) Rn[3 * a + b] = R[3 * a] * Ri[b] + R[3 * a + 1] * Ri[3 + b] + R[3 * a + 2] * Ri[6 + b];
+#pragma unroll
+        for (int a = 0; a < 9; ++a) R[a] = Rn[a];
+      }
+    }
+  }
+#pragma unroll
+  for (int a = 0; a < 3; ++a) r[a] = p[a] - pm[a];
+#pragma unroll
+  for (int i = 0; i < N; ++i) {
+    double t[3], wx[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) t[a] = p[a] - pe[i][a];
+    cross(wv[i], t, wx);
+#pragma unroll
+    for (int a = 0; a < 3; ++a) J[a][N + i] = -(v[i][a] + wx[a]) * rb.rc[i];  // rc holds 1 / r_c here (calib_robot_f64)
+  }
+}
+
+// The LM iteration as one launch, 32 poses (a tile) to a warp. Launch j (1, 2, ...) adds the partial sums
+// that launch j - 1 left at its point, applies the LM rule to it, solves for the next trial point and
+// evaluates residuals, J^T J, J^T r and F there; so a step costs one evaluation and one launch, and an
+// accepted trial's normal equations are at hand. Every block repeats the (short) sums and the solve, which
+// spares a grid barrier; block 0 keeps the state. Partial sums and states alternate between two buffers,
+// because blocks of one launch still read what the last one wrote. A trial point equal to theta needs no
+// evaluation (its cost is F). All sums have a fixed order: a lane adds one entry over its warp's poses in
+// order, the block its warps, every block the blocks' partials in four runs; F adds tile totals t, t + 32,
+// ... on lane t and then the lanes, which the single-block cost kernel repeats.
+// Bound: the FP64 pipe and its latency; 1024 poses are 32 warps on 32 of 608 sub-partitions, each busy with
+// its own poses' instructions. 20 iterations of 1024 poses in FP64: 0.50 ms; as two launches an iteration, the
+// second one block that evaluated the trial cost of all poses on one SM, 2.57 ms.
+constexpr int kCalibThreads = 128, kCalibWarps = kCalibThreads / 32;
+constexpr int kCalibMaxBlocks = 304;  // two per SM; more tiles are looped over
 template <int N> constexpr int calib_nv() { return (2 * N) * (2 * N + 1) / 2 + 2 * N + 1; }
+inline __host__ __device__ int64_t calib_tiles(int64_t K) { return (K + 31) / 32; }
+inline __host__ __device__ int calib_blocks(int64_t K) {
+  const int64_t b = (calib_tiles(K) + kCalibWarps - 1) / kCalibWarps;
+  return (int)(b < kCalibMaxBlocks ? b : kCalibMaxBlocks);
+}
 
 template <typename T, int N> __device__ RobotK<T> calib_robot(RobotK<T> rb, const double* theta) {
 #pragma unroll
   for (int i = 0; i < N; ++i) {
     rb.L[i] = T(theta[i]);
-    rb.rc[i] = T(theta[N + i]);
+    // FP64 rows take 1 / r_c (calib_pose_f64)
+    rb.rc[i] = sizeof(T) == 8 ? T(1.0 / theta[N + i]) : T(theta[N + i]);
     rb.K[i] = T(-2.0 / (3.0 * theta[N + i]));
   }
   return rb;
@@ -449,210 +564,323 @@ __device__ inline double warp_sum_d(double v) {
   return v;
 }
 
+// Residual (and Jacobian) of pose k; zero rows past the last pose.
 template <typename T, int N>
-__global__ void __launch_bounds__(kCalibThreads) k_calib_accum(RobotK<T> rb0, const T* __restrict__ U,
-                                                              const double* __restrict__ Pm, int64_t K,
-                                                              const double* theta, double* part) {
-  constexpr int D = 3 * N, NP = 2 * N, NV = calib_nv<N>();
-  __shared__ double red[kCalibThreads / 32][NV];
-  __shared__ double th[NP];
-  if (threadIdx.x < NP) th[threadIdx.x] = theta[threadIdx.x];
-  __syncthreads();
-  const RobotK<T> rb = calib_robot<T, N>(rb0, th);
-  const int64_t k = (int64_t)blockIdx.x * kCalibThreads + threadIdx.x;
-  T r[3] = {T(0), T(0), T(0)}, J[3][NP];
-#pragma unroll
-  for (int a = 0; a < 3; ++a)
-#pragma unroll
-    for (int x = 0; x < NP; ++x) J[a][x] = T(0);
-  if (k < K) {
-    T u[D];
-#pragma unroll
-    for (int q = 0; q < D; ++q) u[q] = U[q * K + k];
-    const double pm[3] = {Pm[k], Pm[K + k], Pm[2 * K + k]};
-    calib_rows<T, N>(rb, u, pm, r, J);
-  }
-  double Jd[3][NP], rd[3];
+__device__ void calib_load_pose(const RobotK<T>& rb, const T* __restrict__ U, const double* __restrict__ Pm, int64_t K,
+                                int64_t k, T (&r)[3], T (&J)[3][2 * N]) {
+  constexpr int D = 3 * N, NP = 2 * N;
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
-    rd[a] = double(r[a]);
+    r[a] = T(0);
 #pragma unroll
-    for (int x = 0; x < NP; ++x) Jd[a][x] = double(J[a][x]);
+    for (int x = 0; x < NP; ++x) J[a][x] = T(0);
   }
-  const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  int v = 0;
+  if (k >= K) return;
+  T u[D];
 #pragma unroll
-  for (int x = 0; x < NP; ++x)
-#pragma unroll
-    for (int y = 0; y <= x; ++y, ++v) {
-      const double c = warp_sum_d(fma(Jd[2][x], Jd[2][y], fma(Jd[1][x], Jd[1][y], Jd[0][x] * Jd[0][y])));
-      if (lane == 0) red[wid][v] = c;
-    }
-#pragma unroll
-  for (int x = 0; x < NP; ++x, ++v) {
-    const double c = warp_sum_d(fma(Jd[2][x], rd[2], fma(Jd[1][x], rd[1], Jd[0][x] * rd[0])));
-    if (lane == 0) red[wid][v] = c;
-  }
-  {
-    const double c = warp_sum_d(0.5 * fma(rd[2], rd[2], fma(rd[1], rd[1], rd[0] * rd[0])));
-    if (lane == 0) red[wid][v] = c;
-  }
-  __syncthreads();
-  for (int e = threadIdx.x; e < NV; e += kCalibThreads) {
-    double s = red[0][e];
-    for (int w = 1; w < kCalibThreads / 32; ++w) s += red[w][e];
-    part[(int64_t)blockIdx.x * NV + e] = s;
-  }
+  for (int q = 0; q < D; ++q) u[q] = U[q * K + k];
+  const double pm[3] = {Pm[k], Pm[K + k], Pm[2 * K + k]};
+  if constexpr (sizeof(T) == 8) calib_pose_f64<N>(rb, u, pm, r, J);
+  else calib_pose<T, N>(rb, u, pm, r, J);
+}
+// 1/2 |r|^2 of a tile, the same in every lane.
+template <typename T> __device__ double calib_tile_cost(const T (&r)[3]) {
+  const double r0 = double(r[0]), r1 = double(r[1]), r2 = double(r[2]);
+  return warp_sum_d(0.5 * __fma_rn(r2, r2, __fma_rn(r1, r1, __dmul_rn(r0, r0))));
 }
 
-// Cost 1/2 sum |p(u_k; theta) - p_k|^2 (FP32 kinematics, FP64 sum) over all poses by one block.
+// Shared scratch of an evaluation: the poses' rows, column-major with an odd stride, one set per warp.
+template <int N> struct CalibSmem {
+  static constexpr int NC = 2 * N + 1;  // columns: J, then r
+  double row[kCalibWarps][3 * NC][33];
+  double red[kCalibWarps][calib_nv<N>()];
+};
+
+// This block's share of the sums at theta (robot rb): part [NV - 1] of the block, tileF of its tiles.
 template <typename T, int N>
-__device__ double calib_cost_block(const RobotK<T>& rb, const T* __restrict__ U, const double* __restrict__ Pm,
-                                   int64_t K, double* red) {
-  constexpr int D = 3 * N;
-  double lF = 0.0;
-  for (int64_t k = threadIdx.x; k < K; k += blockDim.x) {
-    T u[D];
+__device__ void calib_eval(const RobotK<T>& rb, const T* __restrict__ U, const double* __restrict__ Pm, int64_t K,
+                           double* part, double* tileF, CalibSmem<N>& sm) {
+  constexpr int NP = 2 * N, NV = calib_nv<N>(), NE = NV - 1, PER = (NE + 31) / 32, NC = CalibSmem<N>::NC;
+  const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  int ex[PER], ey[PER];  // this lane's entries: products of columns ex and ey (NP: the residual)
 #pragma unroll
-    for (int q = 0; q < D; ++q) u[q] = U[q * K + k];
-    Chain<T, N> ch;
-    chain_forward(rb, u, ch);
+  for (int m = 0; m < PER; ++m) {
+    int e = lane + 32 * m;
+    e = e < NE ? e : NE - 1;
+    if (e >= NE - NP) {
+      ex[m] = e - (NE - NP);
+      ey[m] = NP;
+    } else {
+      int x = 0;
+      while ((x + 1) * (x + 2) / 2 <= e) ++x;
+      ex[m] = x;
+      ey[m] = e - x * (x + 1) / 2;
+    }
+  }
+  double acc[PER];
+#pragma unroll
+  for (int m = 0; m < PER; ++m) acc[m] = 0.0;
+  const int64_t nt = calib_tiles(K);
+  for (int64_t t = (int64_t)blockIdx.x * kCalibWarps + wid; t < nt; t += (int64_t)gridDim.x * kCalibWarps) {
+    T r[3], J[3][NP];
+    calib_load_pose<T, N>(rb, U, Pm, K, t * 32 + lane, r, J);
+    const double Ft = calib_tile_cost(r);
+    if (lane == 0) tileF[t] = Ft;
+    __syncwarp();
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-      const double ra = double(ch.p[a] - T(Pm[a * K + k]));
-      lF += 0.5 * ra * ra;
+#pragma unroll
+      for (int x = 0; x < NP; ++x) sm.row[wid][a * NC + x][lane] = double(J[a][x]);
+      sm.row[wid][a * NC + NP][lane] = double(r[a]);
+    }
+    __syncwarp();
+#pragma unroll
+    for (int m = 0; m < PER; ++m) {
+      double s0 = 0.0, s1 = 0.0, s2 = 0.0;
+#pragma unroll 8
+      for (int j = 0; j < 32; ++j) {
+        s0 = fma(sm.row[wid][ex[m]][j], sm.row[wid][ey[m]][j], s0);
+        s1 = fma(sm.row[wid][NC + ex[m]][j], sm.row[wid][NC + ey[m]][j], s1);
+        s2 = fma(sm.row[wid][2 * NC + ex[m]][j], sm.row[wid][2 * NC + ey[m]][j], s2);
+      }
+      acc[m] += s0 + s1 + s2;
     }
   }
-  return block_sum(lF, red);
+#pragma unroll
+  for (int m = 0; m < PER; ++m)
+    if (lane + 32 * m < NE) sm.red[wid][lane + 32 * m] = acc[m];
+  __syncthreads();
+  for (int e = threadIdx.x; e < NE; e += kCalibThreads) {
+    double s = sm.red[0][e];
+    for (int w = 1; w < kCalibWarps; ++w) s += sm.red[w][e];
+    part[(int64_t)blockIdx.x * NE + e] = s;
+  }
 }
 
-// state: [0] lambda, [1] nu; part: [nblk][NV]
-template <typename T, int N>
-__global__ void __launch_bounds__(256) k_calib_step(RobotK<T> rb0, const T* __restrict__ U, const double* __restrict__ Pm,
-                                                     int64_t K, int nblk, int it, double lambda0, double* theta,
-                                                     double* state, const double* part, double* hist) {
-  constexpr int NP = 2 * N, NA = NP * (NP + 1) / 2, NV = calib_nv<N>();
-  __shared__ double tot[NV], thn[NP], red[32];
-  __shared__ int ok;
-  for (int e = threadIdx.x; e < NV; e += blockDim.x) {
-    double s = part[e];
-    for (int b = 1; b < nblk; ++b) s += part[(int64_t)b * NV + e];
+// The partial sums of nblk blocks and nt tiles added up into tot [NV] (shared), by a block of kCalibThreads.
+template <int N>
+__device__ void calib_total(const double* part, int nblk, const double* tileF, int64_t nt, double* tot,
+                            CalibSmem<N>& sm) {
+  constexpr int NV = calib_nv<N>(), NE = NV - 1;
+  const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int per = (nblk + kCalibWarps - 1) / kCalibWarps;
+  const int b0 = wid * per, b1 = b0 + per < nblk ? b0 + per : nblk;
+  for (int e = lane; e < NE; e += 32) {
+    double s = 0.0;
+#pragma unroll 4
+    for (int b = b0; b < b1; ++b) s += part[(int64_t)b * NE + e];
+    sm.red[wid][e] = s;
+  }
+  if (wid == kCalibWarps - 1) {
+    double f = 0.0;
+#pragma unroll 4
+    for (int64_t t = lane; t < nt; t += 32) f += tileF[t];
+    f = warp_sum_d(f);
+    if (lane == 0) tot[NV - 1] = f;
+  }
+  __syncthreads();
+  for (int e = threadIdx.x; e < NE; e += kCalibThreads) {
+    double s = sm.red[0][e];
+    for (int w = 1; w < kCalibWarps; ++w) s += sm.red[w][e];
     tot[e] = s;
   }
   __syncthreads();
-  double lam = it == 0 ? lambda0 : state[0], nu = it == 0 ? 2.0 : state[1];
-  double dl[NP], Dg[NP];
-  if (threadIdx.x == 0) {
-    double Ad[NA], iv[NP];
+}
+
+// One warp: the damped step from the sums tot [NV] at theta: trial [NP] (theta where the factorisation
+// fails) and the predicted decrease, the same in every lane; returns whether every pivot was positive.
+template <int N>
+__device__ bool calib_solve(const double* tot, const double* theta, double lam, double* trial, double& pred,
+                            double* col, double* colr) {
+  constexpr int NP = 2 * N, NA = NP * (NP + 1) / 2, SL = AugSlots<NP>::SL;
+  const int lane = threadIdx.x & 31;
+  const AugSlots<NP> sl = aug_slots<NP>(lane);
+  double v[SL];
 #pragma unroll
-    for (int a = 0; a < NA; ++a) Ad[a] = tot[a];
-#pragma unroll
-    for (int q = 0; q < NP; ++q) {
-      Dg[q] = fmax(Ad[tri(q, q)], 1e-12);
-      Ad[tri(q, q)] += lam * Dg[q];
-    }
-    ok = cholesky_packed<NP>(Ad, iv) ? 1 : 0;
-#pragma unroll
-    for (int q = 0; q < NP; ++q) dl[q] = -tot[NA + q];
-    if (ok) {
-      cholesky_solve<NP>(Ad, iv, dl);
-#pragma unroll
-      for (int q = 0; q < NP; ++q) thn[q] = theta[q] + dl[q];
+  for (int s = 0; s < SL; ++s) {
+    v[s] = 0.0;
+    if (!sl.on[s]) continue;
+    const int i = sl.r[s], j = sl.c[s];
+    if (i < NP) {
+      v[s] = tot[tri(i, j)];
+      if (i == j) v[s] += lam * fmax(v[s], 1e-12);
+    } else if (j < NP) {
+      v[s] = -tot[NA + j];
     }
   }
-  __syncthreads();
-  double Fn = 0.0;
-  if (ok) Fn = calib_cost_block<T, N>(calib_robot<T, N>(rb0, thn), U, Pm, K, red);
-  if (threadIdx.x == 0) {
-    const double F = tot[NV - 1];
-    if (ok && Fn < F) {
-      double pred = 0.0;
+  const bool ok = sweep_aug<double, NP>(v, sl, col, colr);
 #pragma unroll
-      for (int q = 0; q < NP; ++q) pred += dl[q] * (lam * Dg[q] * dl[q] - tot[NA + q]);
-      pred *= 0.5;
-      const double rho = (F - Fn) / pred, tt = 2.0 * rho - 1.0;
-      lam *= fmax(1.0 / 3.0, 1.0 - tt * tt * tt);
-      nu = 2.0;
-#pragma unroll
-      for (int q = 0; q < NP; ++q) theta[q] = thn[q];
-    } else {
-      lam *= nu;
-      nu *= 2.0;
-    }
-    state[0] = lam;
-    state[1] = nu;
+  for (int s = 0; s < SL; ++s)
+    if (sl.on[s] && sl.r[s] == NP && sl.c[s] < NP) col[sl.c[s]] = v[s];
+  __syncwarp();
+  double pl = 0.0;
+  if (lane < NP) {
+    const double x = col[lane];
+    trial[lane] = ok ? theta[lane] + x : theta[lane];
+    pl = x * (lam * fmax(tot[tri(lane, lane)], 1e-12) * x - tot[NA + lane]);
   }
-  __syncthreads();
-  if (hist && threadIdx.x < NP) hist[(int64_t)it * NP + threadIdx.x] = theta[threadIdx.x];
+  pred = 0.5 * warp_sum_d(pl);
+  __syncwarp();
+  return ok;
+}
+
+// The LM rule for a trial of cost Fn (taken = whether theta moves to it).
+__device__ inline bool calib_rule(bool ok, double F, double Fn, double pred, double& lam, double& nu) {
+  if (ok && Fn < F) {
+    const double rho = (F - Fn) / pred, tt = 2.0 * rho - 1.0;
+    lam *= fmax(1.0 / 3.0, 1.0 - tt * tt * tt);
+    nu = 2.0;
+    return true;
+  }
+  lam *= nu;
+  nu *= 2.0;
+  return false;
+}
+
+// Workspace of cr_calibrate, in doubles: two states [4 + 2 NP + NV] (lambda, nu, predicted decrease, 0 =
+// evaluated / 1 = trial equal to theta / 2 = failed factorisation, theta, trial, sums at theta), then two
+// sets of partial sums [nblk][NV - 1] and tile costs [tiles].
+template <int N> constexpr int calib_state_len() { return 4 + 4 * N + calib_nv<N>(); }
+inline size_t calibrate_ws_bytes(int n, int64_t K) {
+  const int NP = 2 * n, NV = NP * (NP + 1) / 2 + NP + 1;
+  return (size_t)(2 * ((4 + 2 * NP + NV) + (int64_t)calib_blocks(K) * (NV - 1) + calib_tiles(K))) * sizeof(double);
 }
 
 template <typename T, int N>
-__global__ void __launch_bounds__(256) k_calib_final(RobotK<T> rb0, const T* __restrict__ U, const double* __restrict__ Pm,
-                                                      int64_t K, const double* theta, double* F_out) {
-  constexpr int NP = 2 * N;
-  __shared__ double th[NP], red[32];
-  if (threadIdx.x < NP) th[threadIdx.x] = theta[threadIdx.x];
+__global__ void __launch_bounds__(kCalibThreads) k_calib_eval(RobotK<T> rb0, const T* __restrict__ U,
+                                                             const double* __restrict__ Pm, int64_t K,
+                                                             const double* theta, double* part, double* tileF) {
+  __shared__ CalibSmem<N> sm;
+  __shared__ RobotK<T> rbs;
+  if (threadIdx.x == 0) rbs = calib_robot<T, N>(rb0, theta);
   __syncthreads();
-  const double F = calib_cost_block<T, N>(calib_robot<T, N>(rb0, th), U, Pm, K, red);
-  if (threadIdx.x == 0) *F_out = F;
+  calib_eval<T, N>(rbs, U, Pm, K, part, tileF, sm);
 }
 
-// Sharded calibration: the pieces of k_calib_step as separate launches, so that processes holding
-// shares of the poses can add their partial sums (an all-reduce) in between. Each piece repeats the
-// arithmetic of k_calib_step in the same order, so one process running them equals cr_calibrate.
+// Launch j of the calibration (see above); j = iters + 1 only applies the rule and writes the results.
+template <typename T, int N>
+__global__ void __launch_bounds__(kCalibThreads) k_calib_iter(RobotK<T> rb0, const T* __restrict__ U,
+                                                             const double* __restrict__ Pm, int64_t K, int nblk, int j,
+                                                             int iters, double lambda0, double* theta, double* ws,
+                                                             double* F_out, double* hist) {
+  constexpr int NP = 2 * N, NV = calib_nv<N>(), ST = calib_state_len<N>();
+  __shared__ CalibSmem<N> sm;
+  __shared__ RobotK<T> rbs;
+  __shared__ double tot[NV], cur[NV], th[NP], tr[NP], col[32], colr[32];
+  __shared__ int skip;
+  const int64_t nt = calib_tiles(K);
+  const int64_t pset = (int64_t)nblk * (NV - 1) + nt;
+  const double* old = ws + (j & 1 ? 0 : ST);  // the state that launch j - 1 wrote
+  double* neu = ws + (j & 1 ? ST : 0);
+  const double* part = ws + 2 * ST + (j & 1 ? 0 : pset);
+  double* partn = ws + 2 * ST + (j & 1 ? pset : 0);
+  const int was = j > 1 ? (int)old[3] : 0;  // how the last trial ended
+  if (was == 0) calib_total<N>(part, nblk, part + (int64_t)nblk * (NV - 1), nt, tot, sm);
+  if (threadIdx.x < 32) {
+    const int lane = threadIdx.x;
+    double lam = lambda0, nu = 2.0;
+    bool taken = true;
+    if (j > 1) {
+      lam = old[0];
+      nu = old[1];
+      const double F = old[4 + 2 * NP + NV - 1];
+      taken = calib_rule(was != 2, F, was == 0 ? tot[NV - 1] : F, old[2], lam, nu);
+    }
+    if (lane < NP) th[lane] = j == 1 ? theta[lane] : old[4 + (taken ? NP : 0) + lane];
+    for (int e = lane; e < NV; e += 32) cur[e] = taken ? tot[e] : old[4 + 2 * NP + e];
+    __syncwarp();
+    if (blockIdx.x == 0 && hist && j > 1 && lane < NP) hist[(int64_t)(j - 2) * NP + lane] = th[lane];
+    if (j == iters + 1) {
+      if (blockIdx.x == 0) {
+        if (lane < NP) theta[lane] = th[lane];
+        if (lane == 0) *F_out = cur[NV - 1];
+      }
+      if (lane == 0) skip = 1;
+    } else {
+      double pred;
+      const bool ok = calib_solve<N>(cur, th, lam, tr, pred, col, colr);
+      const bool still = __all_sync(0xffffffffu, lane >= NP || tr[lane < NP ? lane : 0] == th[lane < NP ? lane : 0]);
+      if (lane == 0) skip = !ok ? 2 : (still ? 1 : 0);
+      if (blockIdx.x == 0) {
+        if (lane == 0) {
+          neu[0] = lam;
+          neu[1] = nu;
+          neu[2] = pred;
+          neu[3] = double(!ok ? 2 : (still ? 1 : 0));
+        }
+        if (lane < NP) {
+          neu[4 + lane] = th[lane];
+          neu[4 + NP + lane] = tr[lane];
+        }
+        for (int e = lane; e < NV; e += 32) neu[4 + 2 * NP + e] = cur[e];
+      }
+    }
+  }
+  __syncthreads();
+  if (skip) return;
+  if (threadIdx.x == 0) rbs = calib_robot<T, N>(rb0, tr);
+  __syncthreads();
+  calib_eval<T, N>(rbs, U, Pm, K, partn, partn + (int64_t)nblk * (NV - 1), sm);
+}
+
+// Sharded calibration: the pieces of k_calib_iter as separate launches, so that processes holding
+// shares of the poses can add their partial sums (an all-reduce) in between. Each piece runs the same
+// routines in the same order, so one process running them equals cr_calibrate.
 // sums [NV]: the share's packed J^T J, J^T r and F; state [4]: lambda, nu, ok, pred.
 template <int N>
-__global__ void __launch_bounds__(256) k_calib_sum_parts(int nblk, const double* part, double* sums) {
+__global__ void __launch_bounds__(kCalibThreads) k_calib_sum_parts(int nblk, int64_t nt, const double* part,
+                                                                  const double* tileF, double* sums) {
   constexpr int NV = calib_nv<N>();
-  for (int e = threadIdx.x; e < NV; e += blockDim.x) {
-    double s = part[e];
-    for (int b = 1; b < nblk; ++b) s += part[(int64_t)b * NV + e];
-    sums[e] = s;
-  }
+  __shared__ CalibSmem<N> sm;
+  __shared__ double tot[NV];
+  calib_total<N>(part, nblk, tileF, nt, tot, sm);
+  for (int e = threadIdx.x; e < NV; e += blockDim.x) sums[e] = tot[e];
 }
 
 template <int N>
-__global__ void k_calib_trial(const double* sums, const double* theta, double* state, double* theta_trial) {
-  constexpr int NP = 2 * N, NA = NP * (NP + 1) / 2;
-  if (threadIdx.x != 0) return;
-  const double lam = state[0];
-  double Ad[NA], iv[NP], Dg[NP], dl[NP];
-#pragma unroll
-  for (int a = 0; a < NA; ++a) Ad[a] = sums[a];
-#pragma unroll
-  for (int q = 0; q < NP; ++q) {
-    Dg[q] = fmax(Ad[tri(q, q)], 1e-12);
-    Ad[tri(q, q)] += lam * Dg[q];
+__global__ void __launch_bounds__(32) k_calib_trial(const double* sums, const double* theta, double* state,
+                                                    double* theta_trial) {
+  constexpr int NP = 2 * N, NV = calib_nv<N>();
+  __shared__ double tot[NV], th[NP], tr[NP], col[32], colr[32];
+  for (int e = threadIdx.x; e < NV; e += 32) tot[e] = sums[e];
+  if (threadIdx.x < NP) th[threadIdx.x] = theta[threadIdx.x];
+  __syncwarp();
+  double pred;
+  const bool ok = calib_solve<N>(tot, th, state[0], tr, pred, col, colr);
+  if (threadIdx.x < NP) theta_trial[threadIdx.x] = tr[threadIdx.x];
+  if (threadIdx.x == 0) {
+    state[2] = ok ? 1.0 : 0.0;
+    state[3] = ok ? pred : 0.0;
   }
-  const bool ok = cholesky_packed<NP>(Ad, iv);
-#pragma unroll
-  for (int q = 0; q < NP; ++q) dl[q] = -sums[NA + q];
-  double pred = 0.0;
-  if (ok) {
-    cholesky_solve<NP>(Ad, iv, dl);
-#pragma unroll
-    for (int q = 0; q < NP; ++q) {
-      theta_trial[q] = theta[q] + dl[q];
-      pred += dl[q] * (lam * Dg[q] * dl[q] - sums[NA + q]);
-    }
-    pred *= 0.5;
-  } else {
-#pragma unroll
-    for (int q = 0; q < NP; ++q) theta_trial[q] = theta[q];
-  }
-  state[2] = ok ? 1.0 : 0.0;
-  state[3] = pred;
 }
 
+// F at theta over all poses by one block of 32 warps' worth of tile runs (run l: tiles l, l + 32, ...), added
+// in calib_total's order.
+constexpr int kCalibCostThreads = 256;
 template <typename T, int N>
-__global__ void __launch_bounds__(256) k_calib_cost(RobotK<T> rb0, const T* __restrict__ U, const double* __restrict__ Pm,
-                                                     int64_t K, const double* theta, double* F_out) {
-  constexpr int NP = 2 * N;
-  __shared__ double th[NP], red[32];
-  if (threadIdx.x < NP) th[threadIdx.x] = theta[threadIdx.x];
+__global__ void __launch_bounds__(kCalibCostThreads) k_calib_cost(RobotK<T> rb0, const T* __restrict__ U,
+                                                                 const double* __restrict__ Pm, int64_t K,
+                                                                 const double* theta, double* F_out) {
+  __shared__ RobotK<T> rbs;
+  __shared__ double run[32];
+  if (threadIdx.x == 0) rbs = calib_robot<T, N>(rb0, theta);
   __syncthreads();
-  const double F = calib_cost_block<T, N>(calib_robot<T, N>(rb0, th), U, Pm, K, red);
-  if (threadIdx.x == 0) *F_out = F;
+  const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int64_t nt = calib_tiles(K);
+  for (int l = wid; l < 32; l += kCalibCostThreads / 32) {
+    double f = 0.0;
+    for (int64_t t = l; t < nt; t += 32) {
+      T r[3], J[3][2 * N];
+      calib_load_pose<T, N>(rbs, U, Pm, K, t * 32 + lane, r, J);
+      f += calib_tile_cost(r);
+    }
+    if (lane == 0) run[l] = f;
+  }
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    const double F = warp_sum_d(run[lane]);
+    if (lane == 0) *F_out = F;
+  }
 }
 
 template <int N>
@@ -661,16 +889,9 @@ __global__ void k_calib_accept(const double* sums, const double* F_trial, const 
   constexpr int NP = 2 * N, NV = calib_nv<N>();
   if (threadIdx.x != 0) return;
   double lam = state[0], nu = state[1];
-  const double F = sums[NV - 1], Fn = *F_trial;
-  if (state[2] != 0.0 && Fn < F) {
-    const double rho = (F - Fn) / state[3], tt = 2.0 * rho - 1.0;
-    lam *= fmax(1.0 / 3.0, 1.0 - tt * tt * tt);
-    nu = 2.0;
+  if (calib_rule(state[2] != 0.0, sums[NV - 1], *F_trial, state[3], lam, nu)) {
 #pragma unroll
     for (int q = 0; q < NP; ++q) theta[q] = theta_trial[q];
-  } else {
-    lam *= nu;
-    nu *= 2.0;
   }
   state[0] = lam;
   state[1] = nu;
@@ -811,17 +1032,16 @@ template <typename T, int N> cr_status traj_solve_n(const TrajLaunch& l) {
 }
 
 template <typename T, int N> cr_status calibrate_n(const TrajLaunch& l) {
-  RobotK<T> rb = crh::robot_k<T>(l.robot);
-  const int nblk = (int)((l.K + kCalibThreads - 1) / kCalibThreads);
-  double* state = (double*)l.calib_ws;
-  double* part = state + 2;
+  const RobotK<T> rb = crh::robot_k<T>(l.robot);
+  const int nblk = calib_blocks(l.K);
+  double* ws = (double*)l.calib_ws;
   const T* U = (const T*)l.U;
-  for (int it = 0; it < l.iters; ++it) {
-    k_calib_accum<T, N><<<nblk, kCalibThreads, 0, l.stream>>>(rb, U, l.Pm, l.K, l.theta_dev, part);
-    k_calib_step<T, N><<<1, 256, 0, l.stream>>>(rb, U, l.Pm, l.K, nblk, it, l.lambda0, l.theta_dev, state, part,
-                                                 l.hist_dev);
-  }
-  k_calib_final<T, N><<<1, 256, 0, l.stream>>>(rb, U, l.Pm, l.K, l.theta_dev, l.F_dev);
+  double* part = ws + 2 * calib_state_len<N>();
+  k_calib_eval<T, N><<<nblk, kCalibThreads, 0, l.stream>>>(rb, U, l.Pm, l.K, l.theta_dev, part,
+                                                          part + (int64_t)nblk * (calib_nv<N>() - 1));
+  for (int j = 1; j <= l.iters + 1; ++j)
+    k_calib_iter<T, N><<<j <= l.iters ? nblk : 1, kCalibThreads, 0, l.stream>>>(
+        rb, U, l.Pm, l.K, nblk, j, l.iters, l.lambda0, l.theta_dev, ws, l.F_dev, l.hist_dev);
   return crh::check_launch("cr_calibrate");
 }
 
@@ -829,25 +1049,21 @@ template <typename T, int N> cr_status calib_piece_n(const TrajLaunch& l) {
   RobotK<T> rb = crh::robot_k<T>(l.robot);
   const T* U = (const T*)l.U;
   switch (l.calib_piece) {
-    case 0: {  // partial sums of this share: per-block partials, then their sum in block order
-      const int nblk = (int)((l.K + kCalibThreads - 1) / kCalibThreads);
-      double* part = (double*)l.calib_ws + 2;
-      k_calib_accum<T, N><<<nblk, kCalibThreads, 0, l.stream>>>(rb, U, l.Pm, l.K, l.theta_dev, part);
-      k_calib_sum_parts<N><<<1, 256, 0, l.stream>>>(nblk, part, l.sums);
+    case 0: {  // partial sums of this share: per-block partials, then their total
+      const int nblk = calib_blocks(l.K);
+      double* part = (double*)l.calib_ws + 2 * calib_state_len<N>();
+      double* tileF = part + (int64_t)nblk * (calib_nv<N>() - 1);
+      k_calib_eval<T, N><<<nblk, kCalibThreads, 0, l.stream>>>(rb, U, l.Pm, l.K, l.theta_dev, part, tileF);
+      k_calib_sum_parts<N><<<1, kCalibThreads, 0, l.stream>>>(nblk, calib_tiles(l.K), part, tileF, l.sums);
       break;
     }
     case 1: k_calib_trial<N><<<1, 32, 0, l.stream>>>(l.sums, l.theta_dev, l.state, l.theta_trial); break;
-    case 2: k_calib_cost<T, N><<<1, 256, 0, l.stream>>>(rb, U, l.Pm, l.K, l.theta_dev, l.F_dev); break;
+    case 2:
+      k_calib_cost<T, N><<<1, kCalibCostThreads, 0, l.stream>>>(rb, U, l.Pm, l.K, l.theta_dev, l.F_dev);
+      break;
     default: k_calib_accept<N><<<1, 32, 0, l.stream>>>(l.sums, l.F_trial, l.theta_trial, l.theta_dev, l.state);
   }
   return crh::check_launch("sharded calibration");
-}
-
-// Workspace of cr_calibrate: lambda, nu, then the per-block partial sums.
-inline size_t calibrate_ws_bytes(int n, int64_t K) {
-  const int NP = 2 * n;
-  const int64_t nblk = (K + kCalibThreads - 1) / kCalibThreads;
-  return (size_t)(2 + nblk * (NP * (NP + 1) / 2 + NP + 1)) * sizeof(double);
 }
 
 #define CR_TRAJ_DISPATCH(FN, T, l)         \
