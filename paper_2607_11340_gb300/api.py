@@ -12,15 +12,16 @@ from . import synth
 
 def robot_struct(spec: synth.RobotSpec) -> lib.cr_robot:
     r = lib.cr_robot()
-    r.n, r.m, r.n_b = spec.n, 3, spec.nb
+    n = spec.n
+    r.n, r.m, r.n_b = n, 3, spec.nb
     r.model = lib.CR_MODEL_ARC if spec.is_arc else (lib.CR_MODEL_COUPLED if spec.coupled else lib.CR_MODEL_TENDON)
-    for i in range(spec.n):
-        r.L[i] = spec.L[i]
-        r.r_c[i] = spec.rc
-        r.u_max[i] = spec.umax
-        r.theta_max[i] = spec.thmax
-        if spec.is_arc:
-            r.l_min[i], r.l_max[i] = spec.lmin, spec.lmax
+    r.L[:n] = spec.L
+    r.r_c[:n] = [spec.rc] * n
+    r.u_max[:n] = [spec.umax] * n
+    r.theta_max[:n] = [spec.thmax] * n
+    if spec.is_arc:
+        r.l_min[:n] = [spec.lmin] * n
+        r.l_max[:n] = [spec.lmax] * n
     r.r_body = spec.body_radius
     return r
 
@@ -218,13 +219,13 @@ class IkCost(torch.autograd.Function):
     def forward(ctx, u, L, rc, ctx_data):
         spec, scene, task = ctx_data
         robot = robot_struct(spec)
-        for i in range(spec.n):
-            robot.L[i] = float(L[i])
-            robot.r_c[i] = float(rc[i])
+        n = spec.n
+        robot.L[:n] = L.tolist()[:n]
+        robot.r_c[:n] = rc.tolist()[:n]
         cost = torch.empty(u.shape[1], dtype=u.dtype, device=u.device)
         lib.cr_cost_grad(robot, scene.c, task, u.contiguous(), cost)
         ctx.save_for_backward(u)
-        ctx.robot, ctx.scene, ctx.task, ctx.n = robot, scene, task, spec.n
+        ctx.robot, ctx.scene, ctx.task, ctx.n = robot, scene, task, n
         ctx.param_dtype, ctx.param_device = L.dtype, L.device
         return cost
 
@@ -232,10 +233,14 @@ class IkCost(torch.autograd.Function):
     def backward(ctx, gcost):
         (u,) = ctx.saved_tensors
         gu = torch.empty_like(u)
+        up = gcost.contiguous().to(u.dtype)
+        if not (ctx.needs_input_grad[1] or ctx.needs_input_grad[2]):
+            lib.cr_cost_vjp(ctx.robot, ctx.scene.c, ctx.task, u.contiguous(), up, gu)
+            return gu, None, None, None
         gp = torch.empty(2 * ctx.n, dtype=torch.float64, device=u.device)
         ws = torch.empty((2 * ctx.n, u.shape[1]), dtype=u.dtype, device=u.device)
-        lib.cr_cost_vjp(ctx.robot, ctx.scene.c, ctx.task, u.contiguous(), gcost.contiguous().to(u.dtype), gu, gp, ws)
-        gp = gp.to(ctx.param_device, ctx.param_dtype)
+        lib.cr_cost_vjp(ctx.robot, ctx.scene.c, ctx.task, u.contiguous(), up, gu, gp, ws)
+        gp = gp.to(ctx.param_device).to(ctx.param_dtype)  # to a host dtype on the host: no conversion launch
         return gu, gp[:ctx.n], gp[ctx.n:], None
 
 

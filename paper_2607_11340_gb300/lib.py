@@ -117,6 +117,7 @@ class cr_roadmap(C.Structure):
 
 
 _lib = None
+_torch = None  # the torch module once the library is loaded
 _lock = threading.Lock()
 
 _P = C.c_void_p
@@ -184,10 +185,15 @@ _SIGS = {
 
 def load(path: str | None = None):
     """Load libcrsolver.so (raises if it is missing: build it with build_lib.build())."""
-    global _lib
+    global _lib, _torch
+    if _lib is not None:  # set last, with everything it needs in place
+        return _lib
     with _lock:
         if _lib is not None:
             return _lib
+        import torch
+
+        _torch = torch
         p = path or LIB_PATH
         if not os.path.exists(p):
             raise RuntimeError(f"libcrsolver.so not found at {p}; run paper_2607_11340_gb300.build_lib.build()")
@@ -231,6 +237,9 @@ def _check(st: int):
         raise CrError(st, last_error())
 
 
+# The marshalling below runs once or twice per argument of every call, and a call on one state is bound by
+# it: 16 us of host time for cr_fk, of which torch.cuda.current_stream() (device lookup through the
+# environment, a Stream object) took 6. Pointers go as plain ints, which ctypes takes for a c_void_p.
 def _ptr(t):
     """Device pointer of a tensor (None -> NULL)."""
     if t is None:
@@ -239,24 +248,24 @@ def _ptr(t):
         raise ValueError("CUDA tensor expected")
     if not t.is_contiguous():
         raise ValueError("contiguous tensor expected")
-    return C.c_void_p(t.data_ptr())
+    return t.data_ptr()
 
 
 def _stream(stream=None):
-    import torch
-
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return C.c_void_p(s.cuda_stream)
+    """The given torch stream's handle, or the current stream's of the current device."""
+    if stream is not None:
+        return stream.cuda_stream
+    c = _torch._C
+    return c._cuda_getCurrentRawStream(c._cuda_getDevice())
 
 
 def _dtype_code(t):
-    import torch
-
-    if t.dtype == torch.float32:
+    d = t.dtype
+    if d is _torch.float32:
         return CR_F32
-    if t.dtype == torch.float64:
+    if d is _torch.float64:
         return CR_F64
-    raise ValueError(f"float32/float64 expected, got {t.dtype}")
+    raise ValueError(f"float32/float64 expected, got {d}")
 
 
 # --------------------------------------------------------------------------------------------
