@@ -144,46 +144,54 @@ __device__ double joint_lm_warp(const RobotK<float>& rb, const WeightsK<float>& 
   double* z = reinterpret_cast<double*>(scr + ps.z);
   double* Zg = reinterpret_cast<double*>(scr + ps.zg);
   double lam = lam0, nu = 2.0;
+  // after a rejection the blocks, the gradient and the cost still hold; a step too small to change any
+  // state has the trial cost first computed for that (as in k_path_joint)
+  bool held = false, still_known = false;
+  double F = 0.0, F_still = 0.0;
   cur = 0;
   for (int itn = 0; itn < k_joint; ++itn) {
     float* Xc = cur ? X1 : X0;
     float* Xn = cur ? X0 : X1;
-    double Fl = 0.0;
-    for (int t = lane; t < H; t += 32) {
-      float u[D], gt[D];
+    if (!held) {
+      double Fl = 0.0;
+      for (int t = lane; t < H; t += 32) {
+        float u[D], gt[D];
 #pragma unroll
-      for (int q = 0; q < D; ++q) u[q] = Xc[q * H + t];
-      const TargetK<float> tg = load_target<float>(targets, W, wp0 + t, CR_TASK_IK6);
-      float At[DD];
-      Fl += double(eval_ik_normal<float, float, N, true>(rb, w, CR_TASK_IK6, tg, sph, no, u, At, gt));
+        for (int q = 0; q < D; ++q) u[q] = Xc[q * H + t];
+        const TargetK<float> tg = load_target<float>(targets, W, wp0 + t, CR_TASK_IK6);
+        float At[DD];
+        Fl += double(eval_ik_normal<float, float, N, true>(rb, w, CR_TASK_IK6, tg, sph, no, u, At, gt));
 #pragma unroll
-      for (int e = 0; e < DD; ++e) Af[(size_t)t * DD + e] = At[e];
+        for (int e = 0; e < DD; ++e) Af[(size_t)t * DD + e] = At[e];
 #pragma unroll
-      for (int q = 0; q < D; ++q) g[t * D + q] = double(gt[q]);
-    }
-    __syncwarp();
-    for (int t = lane; t < H; t += 32) {
-#pragma unroll
-      for (int q = 0; q < D; ++q) {
-        const double uq = double(Xc[q * H + t]);
-        double s = 0.0;
-        if (t > 0) {
-          const double dq = uq - double(Xc[q * H + t - 1]);
-          s += ws * dq;
-          Fl += 0.5 * ws * dq * dq;
-        }
-        if (t + 1 < H) s -= ws * (double(Xc[q * H + t + 1]) - uq);
-        g[t * D + q] += s;
+        for (int q = 0; q < D; ++q) g[t * D + q] = double(gt[q]);
       }
+      __syncwarp();
+      for (int t = lane; t < H; t += 32) {
+#pragma unroll
+        for (int q = 0; q < D; ++q) {
+          const double uq = double(Xc[q * H + t]);
+          double s = 0.0;
+          if (t > 0) {
+            const double dq = uq - double(Xc[q * H + t - 1]);
+            s += ws * dq;
+            Fl += 0.5 * ws * dq * dq;
+          }
+          if (t + 1 < H) s -= ws * (double(Xc[q * H + t + 1]) - uq);
+          g[t * D + q] += s;
+        }
+      }
+      F = warp_sum(Fl);
+      held = true;
+      __syncwarp();
     }
-    const double F = warp_sum(Fl);
-    __syncwarp();
     if (!joint_solve_warp<float, D>(Af, g, z, Zg, col, colr, Zs, H, ws, lam)) {
       lam *= nu;
       nu *= 2.0;
       continue;
     }
     double predl = 0.0;
+    bool moved = false;
     for (int t = lane; t < H; t += 32) {
       const double nb = double((t > 0) + (t + 1 < H));
 #pragma unroll
@@ -191,17 +199,26 @@ __device__ double joint_lm_warp(const RobotK<float>& rb, const WeightsK<float>& 
         const double xq = z[t * D + q];
         const double dg = fmax(double(Af[(size_t)t * DD + tri(q, q)]) + ws * nb, 1e-12);
         predl += xq * (lam * dg * xq - g[t * D + q]);
-        Xn[q * H + t] = Xc[q * H + t] + float(xq);
+        const float xc = Xc[q * H + t], xn = xc + float(xq);
+        Xn[q * H + t] = xn;
+        moved = moved || xn != xc;
       }
     }
     const double pred = 0.5 * warp_sum(predl);
+    const bool any = __any_sync(0xffffffffu, moved) != 0;
     __syncwarp();
-    const double Fn = path_cost_warp<N>(rb, w, targets, W, wp0, H, sph, no, ws, Xn);
+    double Fn = F_still;
+    if (any || !still_known) Fn = path_cost_warp<N>(rb, w, targets, W, wp0, H, sph, no, ws, Xn);
+    if (!any) {
+      F_still = Fn;
+      still_known = true;
+    }
     if (Fn < F) {
       const double rho = (F - Fn) / pred, tt = 2.0 * rho - 1.0;
       lam *= fmax(1.0 / 3.0, 1.0 - tt * tt * tt);
       nu = 2.0;
       cur ^= 1;
+      if (any) held = still_known = false;
     } else {
       lam *= nu;
       nu *= 2.0;

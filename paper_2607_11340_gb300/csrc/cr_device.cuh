@@ -759,36 +759,99 @@ CR_HD uint64_t group_sphere_mask(const RobotK<T>& rb, const Chain<T, N>& ch, int
   return out;
 }
 
-// The same sets computed by a warp: lane l tests spheres j0 + l and j0 + l + 32 against every
-// segment and the ballots assemble the masks (identical in all lanes afterwards).
+// Whether point x may be within reach of table entry j (jj relative to j0): the exact test with the reach
+// widened by a relative 1e-5 of the magnitudes involved, far above its rounding, so that no pair the exact
+// test keeps is missing.
+template <typename T> CR_HD bool maybe_near(ObsK<T> ob, int j, const T (&x)[3], T slack = T(0)) {
+  const Sphere4<T> S = ob.s[j];
+  if (ob.prims() && j >= ob.ns) {
+    const PrimK<T>& P = ob.p[j - ob.ns];
+    const T marg = T(1e-5) * (P.reach + c_abs(x[0]) + c_abs(x[1]) + c_abs(x[2]) + c_abs(S.x) + c_abs(S.y) +
+                              c_abs(S.z) + S.reach);
+    return prim_sd(P, x) < P.reach + marg + slack;
+  }
+  const T dx = x[0] - S.x, dy = x[1] - S.y, dz = x[2] - S.z;
+  const T lim = S.reach + slack + T(1e-5) * (c_abs(S.reach) + c_abs(S.x) + c_abs(S.y) + c_abs(S.z));
+  return dx * dx + dy * dy + dz * dz < lim * lim;
+}
+
+// For one state held by a whole warp: hit[i] = the obstacles j0 .. j0 + cnt - 1 (cnt <= 64) that some backbone
+// sample of segment i may be within reach of (a superset of those that are; the same in every lane). The
+// units of work are the groups of kCullGroup samples of all segments: each lane takes a unit (two or more
+// share one and split its obstacles, then its samples), tests its group's ball against all obstacles in a
+// straight run without bit loops, and walks the few that are left over its samples. The order of the rows
+// is the caller's; it only visits segments and obstacles with a hit.
+// What bounds it is one warp's latency: the former form visited the segments one after the other (mid-arc
+// ball, groups, all samples of the segment against the union of the lanes' candidates), about 1100 dependent
+// instructions a state of 4 segments among 32 spheres, half of the evaluation.
 template <typename T, int N>
-__device__ void warp_segment_sphere_masks(const RobotK<T>& rb, const Chain<T, N>& ch, ObsK<T> ob, int j0,
-                                          int cnt, uint64_t (&mask)[N]) {
-  const Sphere4<T>* sph = ob.s;
+__device__ void warp_near_obstacles(const RobotK<T>& rb, const Chain<T, N>& ch, ObsK<T> ob, int j0, int cnt,
+                                    uint64_t (&hit)[N]) {
+  const unsigned FULL = 0xffffffffu;
   const int lane = threadIdx.x & 31;
+  const int G = (rb.nb + kCullGroup - 1) / kCullGroup, units = N * G;
+  int lpu = 32 / units;  // lanes per unit: 1, 2 or 4
+  lpu = lpu >= 4 ? 4 : (lpu >= 2 ? 2 : 1);
+  const int sub = lane & (lpu - 1);
+  const T inb = c_div(T(1), T(rb.nb));
   T lsum = T(0);
 #pragma unroll
-  for (int i = 0; i < N; ++i) lsum += ch.L[i];
+  for (int l = 0; l < N; ++l) lsum += ch.L[l];
 #pragma unroll
-  for (int i = 0; i < N; ++i) {
-    T q[3], m[3], s, c;
-    backbone_point(ch.Rb[i], ch.pb[i], ch.ax[i], ch.ay[i], ch.x[i], ch.L[i], T(0.5), q, m, s, c);
-    const T half = T(0.5) * ch.L[i];
-    uint64_t mk = 0;
+  for (int i = 0; i < N; ++i) hit[i] = 0;
+  for (int u0 = 0; u0 < units; u0 += 32 / lpu) {  // every lane runs every round
+    const int u = u0 + lane / lpu;
+    const bool on = u < units;
+    const int seg = on ? u / G : 0, g = on ? u % G : 0;
+    T Rb[9], pb[3], ax = T(0), ay = T(0), x = T(0), L = T(0);
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const int j = lane + 32 * h;
-      bool hit = false;
-      if (j < cnt) {
-        const Sphere4<T> S = sph[j0 + j];
-        const T dx = m[0] - S.x, dy = m[1] - S.y, dz = m[2] - S.z;
-        const T lim = half + S.reach + T(1e-4) * (lsum + S.reach + c_abs(S.x) + c_abs(S.y) + c_abs(S.z));
-        hit = dx * dx + dy * dy + dz * dz < lim * lim;
+    for (int i = 0; i < N; ++i)
+      if (i == 0 || seg == i) {
+#pragma unroll
+        for (int a = 0; a < 9; ++a) Rb[a] = ch.Rb[i][a];
+#pragma unroll
+        for (int a = 0; a < 3; ++a) pb[a] = ch.pb[i][a];
+        ax = ch.ax[i]; ay = ch.ay[i]; x = ch.x[i]; L = ch.L[i];
       }
-      mk |= (uint64_t)__ballot_sync(0xffffffffu, hit) << (32 * h);
+    const int k0 = g * kCullGroup + 1, k1 = k0 + kCullGroup - 1 < rb.nb ? k0 + kCullGroup - 1 : rb.nb;
+    T q[3], m[3], s, c;
+    backbone_point(Rb, pb, ax, ay, x, L, T(0.5) * T(k0 + k1) * inb, q, m, s, c);
+    const T hb = T(0.5) * T(k1 - k0) * L * inb + T(1e-4) * lsum;
+    unsigned lo = 0, hi = 0;
+#pragma unroll 4
+    for (int j = sub; j < cnt; j += lpu) {
+      const Sphere4<T> S = ob.s[j0 + j];
+      const T dx = m[0] - S.x, dy = m[1] - S.y, dz = m[2] - S.z;
+      const T lim = hb + S.reach + T(1e-4) * (S.reach + c_abs(S.x) + c_abs(S.y) + c_abs(S.z));
+      const unsigned bit = (dx * dx + dy * dy + dz * dz < lim * lim) ? 1u << (j & 31) : 0u;
+      if (j < 32) lo |= bit;
+      else hi |= bit;
     }
-    if (ob.prims() && (mk & ~sphere_bits(ob, j0))) mk = prim_exact_cull(ob, j0, mk, m[0], m[1], m[2], half, lsum);
-    mask[i] = mk;
+    for (int off = 1; off < lpu; off <<= 1) {
+      lo |= __shfl_xor_sync(FULL, lo, off);
+      hi |= __shfl_xor_sync(FULL, hi, off);
+    }
+    uint64_t cand = on ? ((uint64_t)hi << 32) | lo : 0ull;
+    uint64_t mine = 0;
+    if (__any_sync(FULL, cand != 0)) {
+      for (int k = k0 + sub; k <= k1 && cand; k += lpu) {
+        T wp[3];
+        backbone_point(Rb, pb, ax, ay, x, L, T(k) * inb, q, wp, s, c);
+        for (uint64_t bits = cand & ~mine; bits; bits &= bits - 1) {
+          const int jj = __ffsll((long long)bits) - 1;
+          if (maybe_near(ob, j0 + jj, wp)) mine |= 1ull << jj;
+        }
+      }
+      __syncwarp();
+      if (__any_sync(FULL, mine != 0)) {
+#pragma unroll
+        for (int i = 0; i < N; ++i) {
+          const uint64_t v = seg == i ? mine : 0ull;
+          hit[i] |= (uint64_t)__reduce_or_sync(FULL, (unsigned)v);
+          if (cnt > 32) hit[i] |= (uint64_t)__reduce_or_sync(FULL, (unsigned)(v >> 32)) << 32;
+        }
+      }
+    }
   }
 }
 

@@ -63,7 +63,10 @@ __device__ void warm_sweep_warp(const RobotK<T>& rb, const WeightsK<T>& w, const
   for (int t = 1; t < H; ++t) {
     TargetK<T> tg = load_target<T>(wp, PH, base + t, CR_TASK_IK6);
     T lam = lam0, nu = T(2);
-    for (int it = 0; it < k_warm; ++it) warp_lm_step<T, N, OBST>(rb, w, tg, sph, no, u, sl, lam, nu, col, colr, sx, sdg);
+    WarpNormal<T, D> nm;
+    nm.held = false;
+    for (int it = 0; it < k_warm; ++it)
+      if (!warp_lm_step<T, N, OBST>(rb, w, tg, sph, no, u, sl, lam, nu, col, colr, sx, sdg, nm)) break;
 #pragma unroll
     for (int q = 0; q < D; ++q)
       if (q == lane) Xout[q * xstride + t] = u[q];
@@ -367,35 +370,63 @@ __global__ void __launch_bounds__(128) k_path_joint(RobotK<T> rb, WeightsK<T> w,
     return F;
   };
 
+  // A rejected step leaves the path as it was: the blocks, the gradient and the cost still hold and the
+  // next iteration starts at its solve (held); and where the step is so small that every u + step is u,
+  // the trial's cost is the one first computed for that (F_still), whatever the damping.
+  bool held = false, still_known = false;
+  double F = 0.0, F_still = 0.0;
   for (int it = 0; it < a.k_joint; ++it) {
-    // 1. J^T J block and J^T r of every waypoint, plus the smoothness rows' gradient
-    double Fl = 0.0;
-    if (wthr) {
-      T At[DD], gt[D];
-      Fl = double(eval_ik_normal<T, T, N, OBST>(rb, w, CR_TASK_IK6, tg, sph, nob, u, At, gt));
+    // Nothing can follow: the last trial was the path itself and is not below F, and with the growing damping
+    // every further step stays below the states' spacing (the bound of warp_frozen over the whole path).
+    if (held && still_known && !(F_still < F) && lam >= 1.0) {
+      const T nb = T((tid > 0) + (tid + 1 < H));
+      T gn2 = T(0);
+      if (wthr)
 #pragma unroll
-      for (int e = 0; e < DD; ++e) Af[tid * DD + e] = At[e];
-#pragma unroll
-      for (int q = 0; q < D; ++q) {
-        g[tid * D + q] = double(gt[q]);
-        ush[tid * D + q] = u[q];
-      }
-    }
-    __syncthreads();
-    if (wthr) {
-#pragma unroll
-      for (int q = 0; q < D; ++q) {
-        double s = 0.0, uq = double(u[q]);
-        if (tid > 0) {
-          double dq = uq - double(ush[(tid - 1) * D + q]);
-          s += ws * dq;
-          Fl += 0.5 * ws * dq * dq;
+        for (int q = 0; q < D; ++q) {
+          const T gq = T(g[tid * D + q]);
+          gn2 += gq * gq / c_max(Af[tid * DD + tri(q, q)] + a.w_s * nb, T(1e-12));
         }
-        if (tid + 1 < H) s -= ws * (double(ush[(tid + 1) * D + q]) - uq);
-        g[tid * D + q] += s;
-      }
+      const T step = T(4) * c_sqrt(block_sum(gn2, reinterpret_cast<T*>(red)));
+      bool below = true;
+      if (wthr)
+#pragma unroll
+        for (int q = 0; q < D; ++q)
+          below = below && double(step) / lam < double(c_sqrt(c_max(Af[tid * DD + tri(q, q)] + a.w_s * nb, T(1e-12))) *
+                                                       c_fabs(u[q]) * tiny_step<T>());
+      if (__syncthreads_and(below)) break;
     }
-    const double F = block_sum(Fl, red);
+    // 1. J^T J block and J^T r of every waypoint, plus the smoothness rows' gradient
+    if (!held) {
+      double Fl = 0.0;
+      if (wthr) {
+        T At[DD], gt[D];
+        Fl = double(eval_ik_normal<T, T, N, OBST>(rb, w, CR_TASK_IK6, tg, sph, nob, u, At, gt));
+#pragma unroll
+        for (int e = 0; e < DD; ++e) Af[tid * DD + e] = At[e];
+#pragma unroll
+        for (int q = 0; q < D; ++q) {
+          g[tid * D + q] = double(gt[q]);
+          ush[tid * D + q] = u[q];
+        }
+      }
+      __syncthreads();
+      if (wthr) {
+#pragma unroll
+        for (int q = 0; q < D; ++q) {
+          double s = 0.0, uq = double(u[q]);
+          if (tid > 0) {
+            double dq = uq - double(ush[(tid - 1) * D + q]);
+            s += ws * dq;
+            Fl += 0.5 * ws * dq * dq;
+          }
+          if (tid + 1 < H) s -= ws * (double(ush[(tid + 1) * D + q]) - uq);
+          g[tid * D + q] += s;
+        }
+      }
+      F = block_sum(Fl, red);
+      held = true;
+    }
     __syncthreads();
     // 2. FP64 block elimination: from both ends by two warps (from 4 waypoints on), else by warp 0
     if (H >= 4 && blockDim.x >= 64) {
@@ -416,8 +447,12 @@ __global__ void __launch_bounds__(128) k_path_joint(RobotK<T> rb, WeightsK<T> w,
     // 3. trial, gain ratio 1/2 x^T (lambda D x - g), accept
     T un[D];
     double predl = 0.0;
+    bool moved = false;
 #pragma unroll
-    for (int q = 0; q < D; ++q) un[q] = wthr ? u[q] + T(z[tid * D + q]) : u[q];
+    for (int q = 0; q < D; ++q) {
+      un[q] = wthr ? u[q] + T(z[tid * D + q]) : u[q];
+      moved = moved || un[q] != u[q];
+    }
     if (wthr) {
       const double nb = double((tid > 0) + (tid + 1 < H));
 #pragma unroll
@@ -428,14 +463,20 @@ __global__ void __launch_bounds__(128) k_path_joint(RobotK<T> rb, WeightsK<T> w,
       }
     }
     const double pred = 0.5 * block_sum(predl, red);
-    __syncthreads();
-    const double Fn = path_cost(un);
+    const bool any = __syncthreads_or(moved) != 0;
+    double Fn = F_still;
+    if (any || !still_known) Fn = path_cost(un);
+    if (!any) {
+      F_still = Fn;
+      still_known = true;
+    }
     if (Fn < F) {
       double rho = (F - Fn) / pred, tt = 2.0 * rho - 1.0;
       lam *= fmax(1.0 / 3.0, 1.0 - tt * tt * tt);
       nu = 2.0;
 #pragma unroll
       for (int q = 0; q < D; ++q) u[q] = un[q];
+      if (any) held = still_known = false;
     } else {
       lam *= nu;
       nu *= 2.0;

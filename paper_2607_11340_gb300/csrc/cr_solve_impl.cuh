@@ -530,8 +530,10 @@ __global__ void __launch_bounds__(256, 1) k_ik_refine_warp(RobotK<float> rb, Wei
       const TargetK<float> tg = load_target<float>(a.targets, a.P, p, CR_TASK_IK6);
       const AugSlots<D> sl = aug_slots<D>(lane);
       double lam = a.lambda0, nu = 2.0;
+      WarpNormal<float, D> nm;
+      nm.held = false;
       for (int it = 0; it < a.k_final; ++it)
-        warp_lm_step<float, N, true, double>(rb, w, tg, sph, nob, u, sl, lam, nu, col, colr, sx, sdg);
+        if (!warp_lm_step<float, N, true, double>(rb, w, tg, sph, nob, u, sl, lam, nu, col, colr, sx, sdg, nm)) break;
     }
     if (lane == 0) {
 #pragma unroll

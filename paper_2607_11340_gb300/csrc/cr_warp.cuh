@@ -95,24 +95,20 @@ __device__ void warp_row(const AugSlots<D>& sl, T (&A)[AugSlots<D>::SL], T& gq, 
 }
 
 // Full-pose IK residual of one state evaluated by a warp (every lane holds u): returns F (the same
-// in every lane). NORMAL is a run-time (warp-uniform) flag, so that the LM step's two evaluations
-// share one copy of this code. With NORMAL, this lane's slots of J^T J (zero in row D) and, on lane q < D, entry
+// in every lane), this lane's slots of J^T J (zero in row D) and, on lane q < D, entry
 // q of g = J^T r. Rows: pose (6), sum-zero per segment, active tendon bounds, active curvature
 // limits, active clearance pairs (backbone samples split over the lanes).
 template <typename T, int N, bool OBST>
 __device__ T warp_eval(const RobotK<T>& rb, const WeightsK<T>& w, const TargetK<T>& tg, ObsK<T> ob,
-                       int no, const T (&u)[3 * N], const AugSlots<3 * N>& sl, T (&A)[AugSlots<3 * N>::SL], T& gq,
-                       const bool NORMAL) {
+                       int no, const T (&u)[3 * N], const AugSlots<3 * N>& sl, T (&A)[AugSlots<3 * N>::SL], T& gq) {
   constexpr int D = 3 * N, SL = AugSlots<D>::SL;
   const Sphere4<T>* sph = ob.s;
   const int lane = threadIdx.x & 31;
   const bool colq = lane < D;
   const int myl = colq ? lane / 3 : 0, mya = colq ? lane % 3 : 0;
-  if (NORMAL) {
 #pragma unroll
-    for (int s = 0; s < SL; ++s) A[s] = T(0);
-    gq = T(0);
-  }
+  for (int s = 0; s < SL; ++s) A[s] = T(0);
+  gq = T(0);
   Chain<T, N> ch;
   chain_forward(rb, u, ch);
   T r[6], e[3], ang, sn, cs;
@@ -120,7 +116,7 @@ __device__ T warp_eval(const RobotK<T>& rb, const WeightsK<T>& w, const TargetK<
   T F = T(0.5) * (r[0] * r[0] + r[1] * r[1] + r[2] * r[2] + r[3] * r[3] + r[4] * r[4] + r[5] * r[5]);
   // this lane's segment: twist (translational tv, angular tw for the two bending inputs), K, u
   T mtv[2][3], mtw[2][3], myK = T(0), myu = T(0), mysu = T(0);
-  if (NORMAL) {
+  {
     T tv[N][2][3], tw[N][2][3];
     segment_twists(rb, ch, tv, tw);
 #pragma unroll
@@ -182,7 +178,7 @@ __device__ T warp_eval(const RobotK<T>& rb, const WeightsK<T>& w, const TargetK<
       if (lo > T(0)) { F += T(0.5) * w.rho_b * lo * lo; vmask |= 1u << q; }
     }
   }
-  if (NORMAL) {
+  {
 #pragma unroll
     for (int s = 0; s < SL; ++s) {
       const int i = sl.r[s], j = sl.c[s];
@@ -209,11 +205,9 @@ __device__ T warp_eval(const RobotK<T>& rb, const WeightsK<T>& w, const TargetK<
       T th = c_sqrt(ch.x[i]);
       T vk = th - rb.thmax[i];
       F += T(0.5) * w.rho_k * vk * vk;
-      if (NORMAL) {
-        const T ith = c_div(w.sk, th);
-        T jq = (colq && myl == i) ? bend_comp(rb.K[i], ch.ax[i] * ith, ch.ay[i] * ith, mya) : T(0);
-        warp_row<T, D>(sl, A, gq, jq, w.sk * vk);
-      }
+      const T ith = c_div(w.sk, th);
+      T jq = (colq && myl == i) ? bend_comp(rb.K[i], ch.ax[i] * ith, ch.ay[i] * ith, mya) : T(0);
+      warp_row<T, D>(sl, A, gq, jq, w.sk * vk);
     }
   }
   // clearance rows
@@ -221,21 +215,15 @@ __device__ T warp_eval(const RobotK<T>& rb, const WeightsK<T>& w, const TargetK<
   if (OBST && no > 0) {
     const T inb = c_div(T(1), T(rb.nb));
     for (int j0 = 0; j0 < no; j0 += 64) {
-      uint64_t mk[N];
-      warp_segment_sphere_masks(rb, ch, ob, j0, no - j0 < 64 ? no - j0 : 64, mk);
+      uint64_t hit[N];
+      warp_near_obstacles(rb, ch, ob, j0, no - j0 < 64 ? no - j0 : 64, hit);
 #pragma unroll
       for (int ii = 0; ii < N; ++ii) {
-        if (!mk[ii]) continue;
+        const uint64_t um = hit[ii];
+        if (!um) continue;
         for (int k0 = 0; k0 < rb.nb; k0 += 32) {
           const int k = k0 + lane + 1;
           const bool mine = k <= rb.nb;
-          // second level: this lane's group of kCullGroup samples, then the union over the warp
-          const int kg0 = (k - 1) / kCullGroup * kCullGroup + 1;
-          const int kg1 = kg0 + kCullGroup - 1 < rb.nb ? kg0 + kCullGroup - 1 : rb.nb;
-          const uint64_t gml = mine ? group_sphere_mask<T, N>(rb, ch, ii, kg0, kg1, ob, j0, mk[ii]) : 0ull;
-          const uint64_t um = (uint64_t)__reduce_or_sync(0xffffffffu, (unsigned)gml) |
-                              ((uint64_t)__reduce_or_sync(0xffffffffu, (unsigned)(gml >> 32)) << 32);
-          if (!um) continue;
           T q[3], wpt[3], s, c;
           backbone_point(ch.Rb[ii], ch.pb[ii], ch.ax[ii], ch.ay[ii], ch.x[ii], ch.L[ii], T(mine ? k : 1) * inb, q,
                          wpt, s, c);
@@ -264,7 +252,6 @@ __device__ T warp_eval(const RobotK<T>& rb, const WeightsK<T>& w, const TargetK<
               }
             }
             if (act) Fsplit += T(0.5) * w.rho_c * viol * viol;
-            if (!NORMAL) continue;
             unsigned m = __ballot_sync(0xffffffffu, act);
             while (m) {
               const int src = __ffs(m) - 1;
@@ -309,81 +296,131 @@ __device__ T warp_eval(const RobotK<T>& rb, const WeightsK<T>& w, const TargetK<
   return F + Fsplit;
 }
 
+// The normal equations and the cost at the state of a warp's LM iterations, kept from one to the next
+// (`held`; the caller clears it for a new target).
+template <typename T, int D> struct WarpNormal {
+  T A[AugSlots<D>::SL], gq, F;
+  bool held;
+  bool solved;  // the scratch sdg holds this A's damping diagonal
+};
+
+// Relative half spacing of T's numbers below a power of two: |d| < |u| tiny_step gives u + d == u.
+template <typename T> CR_HD constexpr T tiny_step() { return sizeof(T) == 4 ? T(1.0 / 67108864.0) : T(1.0 / 36028797018963968.0); }
+
+// Whether every further iteration is a rejection that leaves u: the step is delta = -(A + lambda D)^-1 g,
+// so with A >= 0 (up to rounding, which lambda >= 1 covers) |delta_q| sqrt(D_q) <= |D^-1/2 g| / lambda.
+// Where twice that bound is below the spacing of u_q for every q, u + delta rounds to u, the trial is
+// the state itself, its cost is F, and lambda only grows. Evaluated by the whole warp; sdg holds D.
+template <typename T, int D, typename V>
+__device__ bool warp_frozen(const T (&u)[D], T gq, const V* sdg, V lam) {
+  const int lane = threadIdx.x & 31;
+  if (!(lam >= V(1))) return false;  // the same in every lane
+  const T dq = lane < D ? T(sdg[lane]) : T(1);
+  T uq = T(0);
+#pragma unroll
+  for (int q = 0; q < D; ++q)
+    if (q == lane) uq = u[q];
+  T gn2 = lane < D ? gq * gq / dq : T(0);
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) gn2 += __shfl_xor_sync(0xffffffffu, gn2, off);
+  // lambda may exceed T's range as a double: the quotient is formed in V
+  const bool still = lane >= D || V(T(2) * c_sqrt(gn2)) / lam < V(c_sqrt(dq) * c_fabs(uq) * tiny_step<T>());
+  return __all_sync(0xffffffffu, still) != 0;
+}
+
 // One damped LM step of the warp's state (Nielsen's lambda update, strict-decrease acceptance).
 // The residual, J^T J and the costs are in the bulk precision T; the damped system is solved, and
-// the gain ratio formed, in V (T for exploration, double for a refinement). Returns the cost after
-// the step. The warp's scratch: col, colr, sx, sdg (D + 1 values of V each).
+// the gain ratio formed, in V (T for exploration, double for a refinement). Returns false once no
+// further iteration can change u (warp_frozen): the caller may stop there. The warp's scratch: col,
+// colr, sx, sdg (D + 1 values of V each; sdg is kept between the iterations on one target).
+// A step costs one solve and one evaluation: the trial is evaluated with its normal equations, which are at
+// hand when it is accepted, and a rejection leaves those of u. What bounds the exploration is the latency of
+// one warp along the path that accepts every step (30 percent of the workload's paths leave their target
+// somewhere and do), where an evaluation without and then one with the normal equations at the same point
+// ran in turn. Converged targets reject 80 to 95 % of the steps from the fifth of 30 on and, with the growing
+// damping, soon leave u as it is: a trial equal to u is not evaluated (it is F), and the rest of the
+// iterations is left out where warp_frozen says that nothing can follow. No value changes by any of this.
 template <typename T, int N, bool OBST, typename V = T>
-__device__ T warp_lm_step(const RobotK<T>& rb, const WeightsK<T>& w, const TargetK<T>& tg, ObsK<T> sph,
-                          int no, T (&u)[3 * N], const AugSlots<3 * N>& sl, V& lam, V& nu, V* col, V* colr, V* sx,
-                          V* sdg) {
+__device__ bool warp_lm_step(const RobotK<T>& rb, const WeightsK<T>& w, const TargetK<T>& tg, ObsK<T> sph,
+                             int no, T (&u)[3 * N], const AugSlots<3 * N>& sl, V& lam, V& nu, V* col, V* colr, V* sx,
+                             V* sdg, WarpNormal<T, 3 * N>& nm) {
   constexpr int D = 3 * N, SL = AugSlots<D>::SL;
   const int lane = threadIdx.x & 31;
-  T A[SL], gq;
-  T ue[D];  // the point evaluated: u (pass 0, with the normal equations), then the trial u + step
+  if (nm.held && nm.solved && warp_frozen<T, D, V>(u, nm.gq, sdg, lam)) return false;
+  T ue[D], A2[SL], gq2;  // the point evaluated (u first, then the trial u + step) and its normal equations
+  V pred = V(0);
 #pragma unroll
   for (int q = 0; q < D; ++q) ue[q] = u[q];
-  T F = T(0), Fn = T(0);
-  V pred = V(0);
-  // One evaluation site for both passes (a loop that is not unrolled): the kernel carries one copy
-  // of the residual code, half the instruction footprint of two inlined evaluations.
+  // One evaluation site for both (a loop that is not unrolled): the kernel carries one copy of the
+  // residual code, half the instruction footprint of two inlined evaluations.
 #pragma unroll 1
-  for (int pass = 0; pass < 2; ++pass) {
-    const T Fe = warp_eval<T, N, OBST>(rb, w, tg, sph, no, ue, sl, A, gq, pass == 0);
-    if (pass == 1) {
-      Fn = Fe;
-      break;
-    }
-    F = Fe;
-    // damped, augmented system [A + lam D | -g]
-    V Av[SL];
+  for (;;) {
+    const bool trial = nm.held;
+    if (trial) {
+      // damped, augmented system [A + lam D | -g]
+      V Av[SL];
 #pragma unroll
-    for (int s = 0; s < SL; ++s) {
-      const int i = sl.r[s], j = sl.c[s];
-      const T gj = __shfl_sync(0xffffffffu, gq, j < D ? j : 0);
-      Av[s] = V(A[s]);
-      if (!sl.on[s]) continue;
-      if (i < D && i == j) {
-        const V dg = c_max(Av[s], V(1e-12));
-        sdg[i] = dg;
-        Av[s] += lam * dg;
-      } else if (i == D) {
-        Av[s] = j < D ? -V(gj) : V(0);
+      for (int s = 0; s < SL; ++s) {
+        const int i = sl.r[s], j = sl.c[s];
+        const T gj = __shfl_sync(0xffffffffu, nm.gq, j < D ? j : 0);
+        Av[s] = V(nm.A[s]);
+        if (!sl.on[s]) continue;
+        if (i < D && i == j) {
+          const V dg = c_max(Av[s], V(1e-12));
+          sdg[i] = dg;
+          Av[s] += lam * dg;
+        } else if (i == D) {
+          Av[s] = j < D ? -V(gj) : V(0);
+        }
       }
+      nm.solved = true;
+      if (!sweep_aug<V, D>(Av, sl, col, colr)) {
+        lam *= nu;
+        nu *= V(2);
+        return true;
+      }
+#pragma unroll
+      for (int s = 0; s < SL; ++s)
+        if (sl.on[s] && sl.r[s] == D && sl.c[s] < D) sx[sl.c[s]] = Av[s];
+      __syncwarp();
+      V predl = V(0);
+      if (lane < D) {
+        const V xq = sx[lane];
+        predl = xq * (lam * sdg[lane] * xq - V(nm.gq));
+      }
+#pragma unroll
+      for (int off = 16; off > 0; off >>= 1) predl += __shfl_xor_sync(0xffffffffu, predl, off);
+      pred = V(0.5) * predl;
+      bool moved = false;
+#pragma unroll
+      for (int q = 0; q < D; ++q) {
+        ue[q] = u[q] + T(sx[q]);
+        moved = moved || ue[q] != u[q];
+      }
+      __syncwarp();
+      if (!moved) break;  // the trial is u itself (the same in every lane): a rejection
     }
-    const bool ok = sweep_aug<V, D>(Av, sl, col, colr);
-    if (!ok) {
-      lam *= nu;
-      nu *= V(2);
-      return F;
+    const T Fe = warp_eval<T, N, OBST>(rb, w, tg, sph, no, ue, sl, A2, gq2);
+    const bool take = !trial || Fe < nm.F;
+    if (trial && !take) break;
+    if (trial) {
+      const V rho = c_div(V(nm.F) - V(Fe), pred), tt = V(2) * rho - V(1);
+      lam *= c_max(V(1) / V(3), V(1) - tt * tt * tt);
+      nu = V(2);
+#pragma unroll
+      for (int q = 0; q < D; ++q) u[q] = ue[q];
     }
+    nm.F = Fe;
+    nm.gq = gq2;
 #pragma unroll
-    for (int s = 0; s < SL; ++s)
-      if (sl.on[s] && sl.r[s] == D && sl.c[s] < D) sx[sl.c[s]] = Av[s];
-    __syncwarp();
-    V predl = V(0);
-    if (lane < D) {
-      const V xq = sx[lane];
-      predl = xq * (lam * sdg[lane] * xq - V(gq));
-    }
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) predl += __shfl_xor_sync(0xffffffffu, predl, off);
-    pred = V(0.5) * predl;
-#pragma unroll
-    for (int q = 0; q < D; ++q) ue[q] = u[q] + T(sx[q]);
-    __syncwarp();
-  }
-  if (Fn < F) {
-    const V rho = c_div(V(F) - V(Fn), pred), tt = V(2) * rho - V(1);
-    lam *= c_max(V(1) / V(3), V(1) - tt * tt * tt);
-    nu = V(2);
-#pragma unroll
-    for (int q = 0; q < D; ++q) u[q] = ue[q];
-    return Fn;
+    for (int s = 0; s < SL; ++s) nm.A[s] = A2[s];
+    nm.held = true;
+    nm.solved = false;
+    if (trial) return true;
   }
   lam *= nu;
   nu *= V(2);
-  return F;
+  return true;
 }
 
 }  // namespace crk
