@@ -732,18 +732,62 @@ CR_HD void segment_sphere_masks(const RobotK<T>& rb, const Chain<T, N>& ch, ObsK
   }
 }
 
+// FP32 form of the same sets (any superset of the pairs within reach is right: the per-sample test
+// decides). One pass over the obstacles serves all segments: an obstacle's own part of the limit,
+// reach + 1e-4 (reach + |c|_1), is formed once, a test is then d^2 - lim^2 and its sign bit is shifted
+// into the mask (10 instructions a pair). Formed per segment with compares and 64-bit shifts a test took
+// about 20, half of the clearance work of a state among 64 spheres. Used where a decision or a cost of its own is
+// the result; the solvers' FP32 evaluations keep the form above, whose results ptxas rounds (fuses)
+// differently when the code beside them changes, which the projected-gradient iterates magnify.
+template <int N>
+CR_HD void segment_sphere_masks_f(const Chain<float, N>& ch, ObsK<float> ob, int j0, int cnt, uint64_t (&mask)[N]) {
+  const Sphere4<float>* sph = ob.s + j0;
+  float lsum = 0.f, m[N][3], hb[N];
+  unsigned lo[N], hi[N];
+#pragma unroll
+  for (int i = 0; i < N; ++i) lsum += ch.L[i];
+#pragma unroll
+  for (int i = 0; i < N; ++i) {
+    float q[3], s, c;
+    backbone_point(ch.Rb[i], ch.pb[i], ch.ax[i], ch.ay[i], ch.x[i], ch.L[i], 0.5f, q, m[i], s, c);
+    hb[i] = fmaf(0.5f, ch.L[i], 1e-4f * lsum);
+    lo[i] = hi[i] = 0u;
+  }
+  auto test = [&](int j, unsigned (&w)[N]) {
+    const Sphere4<float> S = sph[j];
+    const float own = fmaf(1e-4f, S.reach + fabsf(S.x) + fabsf(S.y) + fabsf(S.z), S.reach);
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+      const float dx = m[i][0] - S.x, dy = m[i][1] - S.y, dz = m[i][2] - S.z, lim = hb[i] + own;
+      const float v = fmaf(-lim, lim, fmaf(dx, dx, fmaf(dy, dy, dz * dz)));
+      w[i] = __funnelshift_l(__float_as_uint(v), w[i], 1);  // (w << 1) | sign of v
+    }
+  };
+#pragma unroll 1
+  for (int j = cnt - 1; j >= 32; --j) test(j, hi);
+#pragma unroll 2
+  for (int j = (cnt < 32 ? cnt : 32) - 1; j >= 0; --j) test(j, lo);
+#pragma unroll
+  for (int i = 0; i < N; ++i) {
+    uint64_t mk = ((uint64_t)hi[i] << 32) | lo[i];
+    if (ob.prims() && (mk & ~sphere_bits(ob, j0)))
+      mk = prim_exact_cull(ob, j0, mk, m[i][0], m[i][1], m[i][2], 0.5f * ch.L[i], lsum);
+    mask[i] = mk;
+  }
+}
+
 // Second level: the samples k0..k1 of segment i (arc fractions k / n_b) lie within
 // (k1 - k0) L_i / (2 n_b) of the point at fraction (k0 + k1) / (2 n_b); of the candidates `cand`
 // (bits relative to j0) those within that radius + reach of it, with the same rounding margin.
 constexpr int kCullGroup = 4;  // backbone samples per second-level ball
 template <typename T, int N>
-CR_HD uint64_t group_sphere_mask(const RobotK<T>& rb, const Chain<T, N>& ch, int i, int k0, int k1,
+CR_HD uint64_t group_sphere_mask(int nb, const Chain<T, N>& ch, int i, int k0, int k1,
                                  ObsK<T> ob, int j0, uint64_t cand) {
   const Sphere4<T>* sph = ob.s;
   T lsum = T(0);
 #pragma unroll
   for (int l = 0; l < N; ++l) lsum += ch.L[l];
-  const T inb = c_div(T(1), T(rb.nb));
+  const T inb = c_div(T(1), T(nb));
   T q[3], m[3], s, c;
   backbone_point(ch.Rb[i], ch.pb[i], ch.ax[i], ch.ay[i], ch.x[i], ch.L[i], T(0.5) * T(k0 + k1) * inb, q, m, s, c);
   const T rad = T(0.5) * T(k1 - k0) * ch.L[i] * inb;
@@ -774,6 +818,70 @@ template <typename T> CR_HD bool maybe_near(ObsK<T> ob, int j, const T (&x)[3], 
   const T lim = S.reach + slack + T(1e-5) * (c_abs(S.reach) + c_abs(S.x) + c_abs(S.y) + c_abs(S.z));
   return dx * dx + dy * dy + dz * dz < lim * lim;
 }
+
+// The quicker search for the near samples of one state (FAST). In FP64 it runs on an FP32 copy f of the obstacle
+// table and an FP32 chain of the same bends, down to the samples: it only has to leave a superset, and an FP64
+// instruction holds a sub-partition's unit 64 cycles. The FP32 backbone is within 2e-6 of the FP64 one relative to the
+// robot's length; the margins are 1e-4 (segments, groups) and 1e-5 (samples) of the magnitudes involved.
+template <typename T, int N> struct CullView {
+  CR_HD CullView(const Chain<T, N>&, const Sphere4<float>*) {}
+  CR_HD void masks(const Chain<T, N>& ch, ObsK<T> ob, int j0, int cnt, uint64_t (&mk)[N]) const {
+    segment_sphere_masks_f<N>(ch, ob, j0, cnt, mk);
+  }
+  CR_HD uint64_t samples(int, int, int, uint64_t) const { return 0; }  // FP64 only
+};
+template <int N> struct CullView<double, N> {
+  Chain<float, N> cf;
+  const Sphere4<float>* f;
+  float slack;
+  CR_HD CullView(const Chain<double, N>& ch, const Sphere4<float>* f_) : f(f_), slack(0.f) {
+    float R[9] = {1.f, 0.f, 0.f, 0.f, 1.f, 0.f, 0.f, 0.f, 1.f}, p[3] = {0.f, 0.f, 0.f};
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+      const float ax = float(ch.ax[i]), ay = float(ch.ay[i]), L = float(ch.L[i]), x = ax * ax + ay * ay;
+      float s, c, Ri[9], di[3], t[3], Rn[9];
+      seg_sc(x, s, c);
+      seg_transform(ax, ay, x, s, c, L, Ri, di);
+#pragma unroll
+      for (int a = 0; a < 9; ++a) cf.Rb[i][a] = R[a];
+#pragma unroll
+      for (int a = 0; a < 3; ++a) cf.pb[i][a] = p[a];
+      cf.ax[i] = ax; cf.ay[i] = ay; cf.x[i] = x; cf.L[i] = L;
+      matvec(R, di, t);
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        p[a] += t[a];
+#pragma unroll
+        for (int b = 0; b < 3; ++b) Rn[3 * a + b] = R[3 * a] * Ri[b] + R[3 * a + 1] * Ri[3 + b] + R[3 * a + 2] * Ri[6 + b];
+      }
+#pragma unroll
+      for (int a = 0; a < 9; ++a) R[a] = Rn[a];
+      slack = fmaf(1e-5f, L, slack);
+    }
+  }
+  CR_HD void masks(const Chain<double, N>&, ObsK<double>, int j0, int cnt, uint64_t (&mk)[N]) const {
+    segment_sphere_masks_f<N>(cf, ObsK<float>(f), j0, cnt, mk);
+  }
+  // the samples of segment i (bit k - 1: sample k) that may be within reach of one of the candidates
+  CR_HD uint64_t samples(int nb, int i, int j0, uint64_t cand) const {
+    static_assert(CR_MAX_NB <= 64, "one bit per sample");
+    const ObsK<float> of(f);
+    const float inb = 1.f / float(nb);
+    uint64_t smp = 0;
+    for (int k0 = 1; k0 <= nb; k0 += kCullGroup) {
+      const int k1 = k0 + kCullGroup - 1 < nb ? k0 + kCullGroup - 1 : nb;
+      const uint64_t gm = group_sphere_mask<float, N>(nb, cf, i, k0, k1, of, j0, cand);
+      if (!gm) continue;
+      for (int k = k0; k <= k1; ++k) {
+        float q[3], wp[3], s, c;
+        backbone_point(cf.Rb[i], cf.pb[i], cf.ax[i], cf.ay[i], cf.x[i], cf.L[i], float(k) * inb, q, wp, s, c);
+        for (uint64_t bits = gm; bits; bits &= bits - 1)
+          if (maybe_near(of, j0 + __ffsll((long long)bits) - 1, wp, slack)) smp |= 1ull << (k - 1);
+      }
+    }
+    return smp;
+  }
+};
 
 // For one state held by a whole warp: hit[i] = the obstacles j0 .. j0 + cnt - 1 (cnt <= 64) that some backbone
 // sample of segment i may be within reach of (a superset of those that are; the same in every lane). The
@@ -962,11 +1070,13 @@ CR_HD void self_contact_forward(const RobotK<T>& rb, const WeightsK<T>& w, const
 // they vanish, so callers whose state was just projected onto it skip them (in FP32 the sum-zero
 // row would only add the rounding residue of the projection). OBST compiles the collision rows:
 // the spheres' and, with w.rho_s > 0, the self-contact rows (with_self = false leaves the latter to
-// another thread that evaluates the same state).
-template <typename T, int N, bool OBST, bool GRAD, bool PGRAD, bool BOX = true, int MODEL = CR_MODEL_TENDON>
+// another thread that evaluates the same state). FAST: the quicker search for near samples (CullView; in FP64
+// on the FP32 table f32), whose samples' rows are the same.
+template <typename T, int N, bool OBST, bool GRAD, bool PGRAD, bool BOX = true, int MODEL = CR_MODEL_TENDON,
+          bool FAST = false>
 CR_HD T state_forward(const RobotK<T>& rb, const WeightsK<T>& w, ObsK<T> ob, int no,
                       const T (&u)[3 * N], Chain<T, N>& ch, StateAgg<T, N>& ag, T* coll_out,
-                      bool with_self = true) {
+                      bool with_self = true, const Sphere4<float>* f32 = nullptr) {
   const Sphere4<T>* sph = ob.s;
   chain_forward<T, N, MODEL>(rb, u, ch);
   T coll = T(0);
@@ -979,16 +1089,27 @@ CR_HD T state_forward(const RobotK<T>& rb, const WeightsK<T>& w, ObsK<T> ob, int
   if (OBST && no > 0) {
     const T inb = T(1) / T(rb.nb);
     for (int j0 = 0; j0 < no; j0 += 64) {
-    uint64_t mk[N];
-    segment_sphere_masks(rb, ch, ob, j0, no - j0 < 64 ? no - j0 : 64, mk);
+    uint64_t mk[N], smp[N];
+    (void)smp;
+    if constexpr (FAST) {
+      const CullView<T, N> cv(ch, f32);
+      cv.masks(ch, ob, j0, no - j0 < 64 ? no - j0 : 64, mk);
+      if (sizeof(T) == 8)  // down to the samples
+#pragma unroll
+        for (int i = 0; i < N; ++i) smp[i] = mk[i] ? cv.samples(rb.nb, i, j0, mk[i]) : 0ull;
+    } else {
+      segment_sphere_masks(rb, ch, ob, j0, no - j0 < 64 ? no - j0 : 64, mk);
+    }
 #pragma unroll
     for (int i = 0; i < N; ++i) {
       if (!mk[i]) continue;
+      constexpr bool picked = FAST && sizeof(T) == 8;
       for (int k0 = 1; k0 <= rb.nb; k0 += kCullGroup) {
       const int k1 = k0 + kCullGroup - 1 < rb.nb ? k0 + kCullGroup - 1 : rb.nb;
-      const uint64_t gm = group_sphere_mask<T, N>(rb, ch, i, k0, k1, ob, j0, mk[i]);
+      const uint64_t gm = picked ? mk[i] : group_sphere_mask<T, N>(rb.nb, ch, i, k0, k1, ob, j0, mk[i]);
       if (!gm) continue;
       for (int k = k0; k <= k1; ++k) {
+        if (picked && !((smp[i] >> (k - 1)) & 1ull)) continue;
         T sg = T(k) * inb;
         T q[3], wp[3], s, c;
         backbone_point(ch.Rb[i], ch.pb[i], ch.ax[i], ch.ay[i], ch.x[i], ch.L[i], sg, q, wp, s, c);
@@ -1210,14 +1331,15 @@ CR_HD void pose_tip_force(int kind, const WeightsK<T>& w, const TargetK<T>& tg, 
   }
 }
 
-// Cost (and adjoint) of an IK state: the two phases around the pose rows. BOX as in state_forward.
-template <typename T, int N, bool OBST, bool GRAD, bool PGRAD, bool BOX = true, int MODEL = CR_MODEL_TENDON>
+// Cost (and adjoint) of an IK state: the two phases around the pose rows. BOX and FAST as in state_forward.
+template <typename T, int N, bool OBST, bool GRAD, bool PGRAD, bool BOX = true, int MODEL = CR_MODEL_TENDON,
+          bool FAST = false>
 CR_HD T eval_ik(const RobotK<T>& rb, const WeightsK<T>& w, int kind, const TargetK<T>& tg,
                 ObsK<T> sph, int no, const T (&u)[3 * N], T (&gu)[3 * N], T* gL, T* grc,
-                T* coll_out) {
+                T* coll_out, const Sphere4<float>* f32 = nullptr) {
   Chain<T, N> ch;
   StateAgg<T, N> ag;
-  T F = state_forward<T, N, OBST, GRAD, PGRAD, BOX, MODEL>(rb, w, sph, no, u, ch, ag, coll_out);
+  T F = state_forward<T, N, OBST, GRAD, PGRAD, BOX, MODEL, FAST>(rb, w, sph, no, u, ch, ag, coll_out, true, f32);
   T r[6], e[3], ang, sn, cs;
   pose_rows(kind, w, tg, ch.R, ch.p, r, e, ang, sn, cs);
   F += T(0.5) * (r[0] * r[0] + r[1] * r[1] + r[2] * r[2] + r[3] * r[3] + r[4] * r[4] + r[5] * r[5]);
@@ -1542,7 +1664,7 @@ CR_HD T eval_ik_normal(const RobotK<T>& rb, const WeightsK<T>& w, int kind, cons
       if (!mk[i]) continue;
       for (int k0 = 1; k0 <= rb.nb; k0 += kCullGroup) {
       const int k1 = k0 + kCullGroup - 1 < rb.nb ? k0 + kCullGroup - 1 : rb.nb;
-      const uint64_t gm = group_sphere_mask<T, N>(rb, ch, i, k0, k1, ob, j0, mk[i]);
+      const uint64_t gm = group_sphere_mask<T, N>(rb.nb, ch, i, k0, k1, ob, j0, mk[i]);
       if (!gm) continue;
       for (int k = k0; k <= k1; ++k) {
         T sg = T(k) * inb;
@@ -1923,7 +2045,7 @@ CR_HD bool state_collides(const RobotK<T>& rb, ObsK<T> ob, int no, const T (&u)[
       if (!mk[i]) continue;
       for (int k0 = 1; k0 <= rb.nb; k0 += kCullGroup) {
       const int k1 = k0 + kCullGroup - 1 < rb.nb ? k0 + kCullGroup - 1 : rb.nb;
-      const uint64_t gm = group_sphere_mask<T, N>(rb, ch, i, k0, k1, ob, j0, mk[i]);
+      const uint64_t gm = group_sphere_mask<T, N>(rb.nb, ch, i, k0, k1, ob, j0, mk[i]);
       if (!gm) continue;
       for (int k = k0; k <= k1; ++k) {
         T q[3], wp[3], s, c;

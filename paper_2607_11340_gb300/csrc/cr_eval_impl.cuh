@@ -71,9 +71,17 @@ __global__ void __launch_bounds__(128) k_cost_grad(RobotK<T> rb, WeightsK<T> w, 
   constexpr int D = 3 * N;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   ObsK<T> ob(nullptr);
+  const Sphere4<float>* f32 = nullptr;
   if (OBST) {
     ob = stage_obstacles(spheres, no, prims, np, rb, w.delta, smem_raw);
     __syncthreads();
+    if constexpr (sizeof(T) == 8) {  // the FP32 copy of the table for the broad phase
+      Sphere4<float>* f = reinterpret_cast<Sphere4<float>*>(smem_raw + ((obstacles_smem<T>(no, np) + 15) & ~(size_t)15));
+      for (int j = threadIdx.x; j < no + np; j += blockDim.x)
+        f[j] = Sphere4<float>{float(ob.s[j].x), float(ob.s[j].y), float(ob.s[j].z), float(ob.s[j].reach)};
+      f32 = f;
+      __syncthreads();
+    }
   }
   int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (b >= B) return;
@@ -82,8 +90,8 @@ __global__ void __launch_bounds__(128) k_cost_grad(RobotK<T> rb, WeightsK<T> w, 
   for (int q = 0; q < D; ++q) uu[q] = u[q * B + b];
   TargetK<T> tg = load_target<T>(targets, P, b / S, kind);
   T g[D], gL[N], grc[N], cl;
-  T F = eval_ik<T, N, OBST, (MODE >= 1), (MODE >= 2), true, MODEL>(rb, w, kind, tg, ob, no + np, uu, g, gL, grc,
-                                                                    &cl);
+  T F = eval_ik<T, N, OBST, (MODE >= 1), (MODE >= 2), true, MODEL, true>(rb, w, kind, tg, ob, no + np, uu, g, gL, grc,
+                                                                          &cl, f32);
   if (cost) cost[b] = F;
   if (coll) coll[b] = cl;
   const T up = upstream ? upstream[b] : T(1);  // vector-Jacobian product weight
@@ -197,6 +205,8 @@ template <typename T, int N, int MODEL = CR_MODEL_TENDON> void cost_grad_n(const
   int no = a.scene.n_o, np = a.scene.n_p;
   int mode = a.gp ? 2 : (a.gu ? 1 : 0);
   size_t sm = obstacles_smem<T>(no, np);
+  // FP64: the FP32 table behind it; at most 45 + 4 KB = the 48 KB of a launch without opt-in
+  if (sizeof(T) == 8) sm = ((sm + 15) & ~(size_t)15) + (size_t)(no + np) * sizeof(Sphere4<float>);
   unsigned g = grid_of(a.B, 128);
 #define CR_CG(OB, MO)                                                                              \
   k_cost_grad<T, N, OB, MO, MODEL><<<g, 128, sm, a.stream>>>(rb, w, a.task.kind, a.task.targets,   \

@@ -116,12 +116,12 @@ __device__ int prm_class32(const RobotK<float>& rb, const PrmSph& s, int no, con
   bool unsure = false;
   for (int j0 = 0; j0 < no; j0 += 64) {
     uint64_t mk[N];
-    segment_sphere_masks(rb, ch, ObsK<float>(s.hi), j0, no - j0 < 64 ? no - j0 : 64, mk);
+    segment_sphere_masks_f<N>(ch, ObsK<float>(s.hi), j0, no - j0 < 64 ? no - j0 : 64, mk);
     for (int i = 0; i < N; ++i) {
       if (!mk[i]) continue;
       for (int k0 = 1; k0 <= rb.nb; k0 += kCullGroup) {
         const int k1 = k0 + kCullGroup - 1 < rb.nb ? k0 + kCullGroup - 1 : rb.nb;
-        const uint64_t gm = group_sphere_mask<float, N>(rb, ch, i, k0, k1, s.hi, j0, mk[i]);
+        const uint64_t gm = group_sphere_mask<float, N>(rb.nb, ch, i, k0, k1, s.hi, j0, mk[i]);
         if (!gm) continue;
         for (int k = k0; k <= k1; ++k) {
           float q[3], wp[3], sn, cs;

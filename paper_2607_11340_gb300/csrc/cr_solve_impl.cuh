@@ -330,11 +330,12 @@ __global__ void __launch_bounds__(256) k_ik_select(IkArgs<T> a, StageOut<T> so, 
 }
 
 // FP64 acceptance of one state: cost, pose errors, limit and clearance flags.
-template <int N, bool OBST, int MODEL = CR_MODEL_TENDON>
+// CULL: the search for near samples runs on the FP32 obstacle table f32 (CullView).
+template <int N, bool OBST, int MODEL = CR_MODEL_TENDON, bool CULL = false>
 CR_HD double accept_fp64(const RobotK<double>& rb, const WeightsK<double>& w, int kind,
                          const TargetK<double>& tg, ObsK<double> ob, int no,
                          const double (&u)[3 * N], double lim_tol, double& pos, double& rot,
-                         unsigned char& flags) {
+                         unsigned char& flags, const Sphere4<float>* f32 = nullptr) {
   const Sphere4<double>* sph = ob.s;
   double dummy[3 * N];
   double F = eval_ik<double, N, OBST, false, false, true, MODEL>(rb, w, kind, tg, ob, no, u, dummy, nullptr, nullptr,
@@ -370,7 +371,36 @@ CR_HD double accept_fp64(const RobotK<double>& rb, const WeightsK<double>& w, in
   }
   // clearance without the margin (radius r_o + r_body); the broad phase uses the larger reach
   bool free = true;
-  if (OBST && no > 0) {
+  if (CULL && OBST && no > 0) {
+    const double inb = 1.0 / rb.nb;
+    const CullView<double, N> cv(ch, f32);
+    for (int j0 = 0; j0 < no && free; j0 += 64) {
+      uint64_t mk[N];
+      cv.masks(ch, ob, j0, no - j0 < 64 ? no - j0 : 64, mk);
+#pragma unroll
+      for (int i = 0; i < N; ++i) {
+        if (!mk[i] || !free) continue;
+        for (uint64_t smp = cv.samples(rb.nb, i, j0, mk[i]); smp && free; smp &= smp - 1) {
+          double q[3], wp[3], s, c;
+          backbone_point(ch.Rb[i], ch.pb[i], ch.ax[i], ch.ay[i], ch.x[i], ch.L[i], __ffsll((long long)smp) * inb, q, wp, s,
+                         c);
+          for (uint64_t bits = mk[i]; bits; bits &= bits - 1) {
+            const int j = j0 + __ffsll((long long)bits) - 1;
+            if (ob.prims() && j >= ob.ns) {
+              const PrimK<double>& P = ob.p[j - ob.ns];
+              double viol, nv[3];
+              if (prim_active(P, wp, P.reach - w.delta, viol, nv)) { free = false; break; }
+              continue;
+            }
+            double ddx = wp[0] - sph[j].x, ddy = wp[1] - sph[j].y, ddz = wp[2] - sph[j].z;
+            double r = sph[j].reach - w.delta;
+            if (ddx * ddx + ddy * ddy + ddz * ddz < r * r) { free = false; break; }
+          }
+        }
+      }
+    }
+  }
+  if (!CULL && OBST && no > 0) {
     const double inb = 1.0 / rb.nb;
     for (int j0 = 0; j0 < no && free; j0 += 64) {
       uint64_t mk[N];
@@ -380,7 +410,7 @@ CR_HD double accept_fp64(const RobotK<double>& rb, const WeightsK<double>& w, in
         if (!mk[i] || !free) continue;
         for (int k0 = 1; k0 <= rb.nb && free; k0 += kCullGroup) {
           const int k1 = k0 + kCullGroup - 1 < rb.nb ? k0 + kCullGroup - 1 : rb.nb;
-          const uint64_t gm = group_sphere_mask<double, N>(rb, ch, i, k0, k1, ob, j0, mk[i]);
+          const uint64_t gm = group_sphere_mask<double, N>(rb.nb, ch, i, k0, k1, ob, j0, mk[i]);
           for (int k = k0; k <= k1 && gm && free; ++k) {
             double q[3], wp[3], s, c;
             backbone_point(ch.Rb[i], ch.pb[i], ch.ax[i], ch.ay[i], ch.x[i], ch.L[i], k * inb, q, wp, s, c);
@@ -516,9 +546,9 @@ __global__ void __launch_bounds__(256, 1) k_ik_refine_warp(RobotK<float> rb, Wei
   double* sx = colr + 32;
   double* sdg = sx + 32;
   const int64_t p = blockIdx.x;
-  const ObsK<double> sphd = stage_problem_obstacles(a, p, rbd, wd.delta, smem_raw);
   const ObsK<float> sph =
       stage_problem_obstacles(a, p, rb, w.delta, smem_raw + ((obstacles_smem<double>(a.no, a.np) + 15) & ~(size_t)15));
+  const ObsK<double> sphd = stage_problem_obstacles(a, p, rbd, wd.delta, smem_raw);
   __syncthreads();
   const int64_t PK = a.P * a.K;
   {
@@ -552,7 +582,8 @@ __global__ void __launch_bounds__(256, 1) k_ik_refine_warp(RobotK<float> rb, Wei
     unsigned char flags = 0;
     if (isfinite(ud[0])) {
       const TargetK<double> tgd = load_target<double>(a.targets, a.P, p, CR_TASK_IK6);
-      F = accept_fp64<N, true>(rbd, wd, CR_TASK_IK6, tgd, sphd, nob, ud, a.lim_tol, pos, rot, flags);
+      F = accept_fp64<N, true, CR_MODEL_TENDON, true>(rbd, wd, CR_TASK_IK6, tgd, sphd, nob, ud, a.lim_tol, pos, rot, flags,
+                                                      sph.s);
     }
 #pragma unroll
     for (int q = 0; q < D; ++q) a.cand_u64[q * PK + c] = ud[q];
