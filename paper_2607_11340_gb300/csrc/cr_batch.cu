@@ -216,7 +216,18 @@ cr_status make_layout(const cr_batch_item* items, int64_t N, const cr_batch_para
       const int bps = std::max(1, blocks_per_sm(n, ph, rb));
       const int64_t want = (work[ph] + crk::kBatchWarps - 1) / crk::kBatchWarps;
       L.grid[n - 1].g[ph] = work[ph] == 0 ? 0 : (int)std::min<int64_t>(want, (int64_t)bps * n_sm);
+      L.grid[n - 1].warps[ph] = crk::kBatchWarps;
+      // refine and exploration of few items: as few warps to a block as put one block on every SM (the warps of
+      // one SM share its instruction cache, and these phases run far more code than it holds)
+      if ((ph == 1 || ph == 2) && work[ph] > 0 && want < n_sm) {
+        const int wpb = (int)((work[ph] + n_sm - 1) / n_sm);
+        L.grid[n - 1].warps[ph] = wpb;
+        L.grid[n - 1].g[ph] = (int)((work[ph] + wpb - 1) / wpb);
+      }
     }
+    // joint phase of few path items: a block to an item, as long as all of them are resident at once (two
+    // blocks of 255 registers a thread to an SM); more items keep the chip busy with a warp to each
+    L.grid[n - 1].joint_blocks = npath > 0 && npath <= 2 * (int64_t)n_sm ? (int)npath : 0;
     L.workers += (int64_t)L.grid[n - 1].g[0] * crk::kBatchWarps;
   }
   L.item_begin[CR_MAX_SEG] = (int64_t)L.items.size();

@@ -506,10 +506,228 @@ __global__ void __maxnreg__(255)
   }
 }
 
+// The joint LM of joint_lm_warp by a block of four warps, a waypoint to a thread (H <= 128): the evaluations of
+// all waypoints run side by side; everything else, the sums over the waypoints in the warp form's order
+// among it, is warp 0's, so that both forms give the same values. fe: 128 doubles, ctl: 4 ints (shared).
+template <int N>
+__device__ double joint_lm_block(const RobotK<float>& rb, const WeightsK<float>& w, const double* targets, int64_t W,
+                                 int64_t wp0, int H, const Sphere4<float>* sph, int no, int k_joint, double lam0,
+                                 double ws, unsigned char* scr, double* col, double* colr, double* Zs, double* fe,
+                                 int* ctl, int& cur) {
+  constexpr int D = 3 * N, DD = D * (D + 1) / 2;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, tw = threadIdx.x;
+  const PathScratch ps = path_scratch(D, H);
+  float* X0 = reinterpret_cast<float*>(scr + ps.x0);
+  float* X1 = reinterpret_cast<float*>(scr + ps.x1);
+  float* Af = reinterpret_cast<float*>(scr + ps.af);
+  double* g = reinterpret_cast<double*>(scr + ps.g);
+  double* z = reinterpret_cast<double*>(scr + ps.z);
+  double* Zg = reinterpret_cast<double*>(scr + ps.zg);
+  // this thread's waypoint of the states X: its cost into fe
+  auto eval_cost = [&](const float* X) {
+    if (tw >= H) return;
+    float u[D], dummy[D];
+#pragma unroll
+    for (int q = 0; q < D; ++q) u[q] = X[q * H + tw];
+    const TargetK<float> tg = load_target<float>(targets, W, wp0 + tw, CR_TASK_IK6);
+    fe[tw] = double(eval_ik<float, N, true, false, false>(rb, w, CR_TASK_IK6, tg, sph, no, u, dummy, nullptr, nullptr,
+                                                          nullptr));
+  };
+  // warp 0: the sum of path_cost_warp over the costs in fe
+  auto sum_cost = [&](const float* X) {
+    double Fl = 0.0;
+    for (int t = lane; t < H; t += 32) {
+      Fl += fe[t];
+      if (t >= 1) {
+#pragma unroll
+        for (int q = 0; q < D; ++q) {
+          const double dq = double(X[q * H + t]) - double(X[q * H + t - 1]);
+          Fl += 0.5 * ws * dq * dq;
+        }
+      }
+    }
+    return warp_sum(Fl);
+  };
+  double lam = lam0, nu = 2.0, F = 0.0, F_still = 0.0;  // warp 0's (as in joint_lm_warp)
+  bool held = false, still_known = false;
+  cur = 0;
+  for (int itn = 0; itn < k_joint; ++itn) {
+    float* Xc = cur ? X1 : X0;
+    float* Xn = cur ? X0 : X1;
+    if (!held && tw < H) {
+      float u[D], gt[D];
+#pragma unroll
+      for (int q = 0; q < D; ++q) u[q] = Xc[q * H + tw];
+      const TargetK<float> tg = load_target<float>(targets, W, wp0 + tw, CR_TASK_IK6);
+      float At[DD];
+      fe[tw] = double(eval_ik_normal<float, float, N, true>(rb, w, CR_TASK_IK6, tg, sph, no, u, At, gt));
+#pragma unroll
+      for (int e = 0; e < DD; ++e) Af[(size_t)tw * DD + e] = At[e];
+#pragma unroll
+      for (int q = 0; q < D; ++q) g[tw * D + q] = double(gt[q]);
+    }
+    __syncthreads();
+    double pred = 0.0;
+    bool any = false;
+    if (wid == 0) {
+      if (!held) {
+        double Fl = 0.0;
+        for (int t = lane; t < H; t += 32) Fl += fe[t];
+        for (int t = lane; t < H; t += 32) {
+#pragma unroll
+          for (int q = 0; q < D; ++q) {
+            const double uq = double(Xc[q * H + t]);
+            double s = 0.0;
+            if (t > 0) {
+              const double dq = uq - double(Xc[q * H + t - 1]);
+              s += ws * dq;
+              Fl += 0.5 * ws * dq * dq;
+            }
+            if (t + 1 < H) s -= ws * (double(Xc[q * H + t + 1]) - uq);
+            g[t * D + q] += s;
+          }
+        }
+        F = warp_sum(Fl);
+        __syncwarp();
+      }
+      const bool ok = joint_solve_warp<float, D>(Af, g, z, Zg, col, colr, Zs, H, ws, lam);
+      if (ok) {
+        double predl = 0.0;
+        bool moved = false;
+        for (int t = lane; t < H; t += 32) {
+          const double nb = double((t > 0) + (t + 1 < H));
+#pragma unroll
+          for (int q = 0; q < D; ++q) {
+            const double xq = z[t * D + q];
+            const double dg = fmax(double(Af[(size_t)t * DD + tri(q, q)]) + ws * nb, 1e-12);
+            predl += xq * (lam * dg * xq - g[t * D + q]);
+            const float xc = Xc[q * H + t], xn = xc + float(xq);
+            Xn[q * H + t] = xn;
+            moved = moved || xn != xc;
+          }
+        }
+        pred = 0.5 * warp_sum(predl);
+        any = __any_sync(0xffffffffu, moved) != 0;
+      }
+      if (lane == 0) ctl[0] = !ok ? 0 : (any || !still_known ? 2 : 1);  // 2: the trial's cost is wanted
+    }
+    __syncthreads();
+    const int what = ctl[0];
+    if (what == 2) eval_cost(Xn);
+    __syncthreads();
+    if (wid == 0) {
+      held = true;
+      bool flip = false;
+      if (what == 0) {
+        lam *= nu;
+        nu *= 2.0;
+      } else {
+        const double Fn = what == 2 ? sum_cost(Xn) : F_still;
+        if (!any) {
+          F_still = Fn;
+          still_known = true;
+        }
+        if (Fn < F) {
+          const double rho = (F - Fn) / pred, tt = 2.0 * rho - 1.0;
+          lam *= fmax(1.0 / 3.0, 1.0 - tt * tt * tt);
+          nu = 2.0;
+          flip = true;
+          if (any) held = still_known = false;
+        } else {
+          lam *= nu;
+          nu *= 2.0;
+        }
+      }
+      if (lane == 0) {
+        ctl[1] = held;
+        ctl[2] = flip;
+      }
+    }
+    __syncthreads();
+    held = ctl[1] != 0;
+    if (ctl[2]) cur ^= 1;
+  }
+  const float* X = cur ? X1 : X0;
+  eval_cost(X);
+  __syncthreads();
+  return wid == 0 ? sum_cost(X) : 0.0;
+}
+
+// Phase 4 with a block to a path item, for batches whose path items of one segment count are few (see
+// batch_joint_blocks): one warp's share of a long path, 128 waypoints in four rounds of evaluations, sets the
+// time of such a batch (63 of 116 ms for 192 mixed items, 6 segments).
+template <int N>
+__global__ void __maxnreg__(255)
+    k_batch_joint_block(RobotK<float> rb, WeightsK<float> w, RobotK<double> rbd, WeightsK<double> wd, BatchArgs a) {
+  constexpr int D = 3 * N;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ int item_s, ctl[4];
+  __shared__ double fe[CR_BATCH_MAX_H];
+  const int wid = threadIdx.x >> 5, tw = threadIdx.x;
+  BatchSmem b;  // warp 0's region, shared by the block
+  b.sph = reinterpret_cast<Sphere4<float>*>(smem_raw);
+  b.sphd = reinterpret_cast<Sphere4<double>*>(smem_raw + 1024);
+  b.col = reinterpret_cast<double*>(smem_raw + 3584);
+  b.colr = b.col + 32;
+  b.Zs = b.colr + 32;
+  unsigned char* scr = a.scratch + (size_t)blockIdx.x * a.scratch_stride;
+  for (;;) {
+    if (tw == 0) item_s = atomicAdd(a.head + 3, 1);
+    __syncthreads();
+    const int i = item_s;
+    __syncthreads();
+    if (i >= a.n_items) break;
+    const BatchItemK it = a.items[i];
+    if (!batch_is_path(it)) continue;
+    const float* Xi = a.xbuf + it.xs;
+    if (!c_finite(__ldcg(Xi))) continue;
+    if (wid == 0) batch_spheres(a, it, rb, w, b.sph);
+    if (wid == 1) batch_spheres_d(a, it, rbd, wd, b.sphd);
+    const int H = it.H;
+    const PathScratch ps = path_scratch(D, H);
+    float* X0 = reinterpret_cast<float*>(scr + ps.x0);
+    for (int e = tw; e < D * H; e += 32 * kBatchWarps) X0[e] = __ldcg(Xi + e);
+    __syncthreads();
+    int cur = 0;
+    const double Ff = joint_lm_block<N>(rb, w, a.targets, a.W, it.wp, H, b.sph, it.no, a.k_joint, a.lambda0, a.w_s, scr,
+                                        b.col, b.colr, b.Zs, fe, ctl, cur);
+    const float* X = reinterpret_cast<const float*>(scr + (cur ? ps.x1 : ps.x0));
+    bool succ = true, lim = true, free = true;
+    if (tw < H) {
+      double uw[D];
+#pragma unroll
+      for (int q = 0; q < D; ++q) {
+        uw[q] = double(X[q * H + tw]);
+        a.u_out[it.st + q * H + tw] = uw[q];
+      }
+      const TargetK<double> tgd = load_target<double>(a.targets, a.W, it.wp + tw, CR_TASK_IK6);
+      double pw, rw;
+      unsigned char f;
+      accept_fp64<N, true>(rbd, wd, CR_TASK_IK6, tgd, b.sphd, it.no, uw, a.lim_tol, pw, rw, f);
+      a.pos[it.wp + tw] = pw;
+      a.rot[it.wp + tw] = rw;
+      lim = f & 1;
+      free = f & 2;
+      succ = pw <= a.pos_tol && rw <= a.rot_tol;
+    }
+    lim = __syncthreads_and(lim);
+    free = __syncthreads_and(free);
+    succ = __syncthreads_and(succ) && lim && free;
+    if (tw == 0) {
+      a.cost[it.item] = Ff;
+      a.flags[it.item] = (unsigned char)((succ ? 1 : 0) | (lim ? 2 : 0) | (free ? 4 : 0));
+      a.t_done[it.item] = global_ns() - *a.t0;
+    }
+    __syncthreads();
+  }
+}
+
 // Host wrappers per segment count (each instantiated in its own translation unit). phase: 0 seeds,
 // 1 refine, 2 exploration, 3 joint.
 struct BatchGrids {
-  int g[4];
+  int g[4];      // blocks
+  int warps[4];  // warps per block
+  int joint_blocks;  // > 0: the joint phase runs with a block to an item, on so many blocks
 };
 template <int N> cr_status batch_prepare(size_t smem) {
   cudaError_t e = cudaFuncSetAttribute(k_batch_seeds<N, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -521,6 +739,8 @@ template <int N> cr_status batch_prepare(size_t smem) {
     e = cudaFuncSetAttribute(k_batch_warm<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(k_batch_joint<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k_batch_joint_block<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return crh::fail(CR_ECUDA, "k_batch phases <%d>: %s", N, cudaGetErrorString(e));
   return CR_OK;
 }
@@ -546,14 +766,16 @@ template <int N> cr_status batch_launch(const cr_robot& family, const cr_weights
   const WeightsK<float> w = crh::weights_k<float>(wts);
   const RobotK<double> rbd = crh::robot_k<double>(r);
   const WeightsK<double> wd = crh::weights_k<double>(wts);
-  const unsigned bs = 32 * kBatchWarps;
+  // a warp's share of the shared memory is kBatchWarpSmem whatever the block's size
+  const auto sm = [&](int ph) { return smem / kBatchWarps * gr.warps[ph]; };
   if (gr.g[0] > 0) {
-    if (rb_seeds == 0) k_batch_seeds<N, 0><<<gr.g[0], bs, smem, s>>>(rb, w, a);
-    else k_batch_seeds<N, 1><<<gr.g[0], bs, smem, s>>>(rb, w, a);
+    if (rb_seeds == 0) k_batch_seeds<N, 0><<<gr.g[0], 32 * gr.warps[0], sm(0), s>>>(rb, w, a);
+    else k_batch_seeds<N, 1><<<gr.g[0], 32 * gr.warps[0], sm(0), s>>>(rb, w, a);
   }
-  if (gr.g[1] > 0) k_batch_refine<N><<<gr.g[1], bs, smem, s>>>(rb, w, rbd, wd, a);
-  if (gr.g[2] > 0) k_batch_warm<N><<<gr.g[2], bs, smem, s>>>(rb, w, a);
-  if (gr.g[3] > 0) k_batch_joint<N><<<gr.g[3], bs, smem, s>>>(rb, w, rbd, wd, a);
+  if (gr.g[1] > 0) k_batch_refine<N><<<gr.g[1], 32 * gr.warps[1], sm(1), s>>>(rb, w, rbd, wd, a);
+  if (gr.g[2] > 0) k_batch_warm<N><<<gr.g[2], 32 * gr.warps[2], sm(2), s>>>(rb, w, a);
+  if (gr.joint_blocks > 0) k_batch_joint_block<N><<<gr.joint_blocks, 32 * kBatchWarps, sm(3), s>>>(rb, w, rbd, wd, a);
+  else if (gr.g[3] > 0) k_batch_joint<N><<<gr.g[3], 32 * gr.warps[3], sm(3), s>>>(rb, w, rbd, wd, a);
   return crh::check_launch("k_batch phases");
 }
 
