@@ -1796,14 +1796,23 @@ CR_HD T eval_ik_normal(const RobotK<T>& rb, const WeightsK<T>& w, int kind, cons
 // relative error e (<= 2^-22 with the rounding of d to float) becomes e^2 after one step and e^4
 // after two, below FP64 rounding, so the result is within a few ulp of 1/d. Four FMAs on the FP64
 // pipe instead of the longer division sequence. Outside the single-precision normal range the
-// division is taken.
+// division is taken. The range check, the rounding of d to float (to nearest, ties to even) and the widening
+// of the seed are done on the bits, with the integer pipes: as FP64 comparisons and conversions they held the
+// FP64 pipe, which bounds the block solves, for as long as the four FMAs do (path following, 512 x 64
+// waypoints: 35.1 -> 32.3 ms).
 CR_HD double recip_nr(double d) {
-  const double ad = d < 0.0 ? -d : d;
-  if (!(ad > 1e-37 && ad < 1e37)) return 1.0 / d;
-  const float f = __double2float_rn(d);
+  const uint64_t b = (uint64_t)__double_as_longlong(d), ab = b & 0x7fffffffffffffffull;
+  const uint64_t lo = (uint64_t)__double_as_longlong(1e-37), hi = (uint64_t)__double_as_longlong(1e37);
+  if (!(ab > lo && ab < hi)) return 1.0 / d;  // NaN and infinity are above hi
+  const unsigned sign = (unsigned)(b >> 32) & 0x80000000u;
+  // exponent bias 1023 -> 127: 896 at the float's exponent position; d and 1/d are normal floats
+  const uint64_t rn = ((ab + 0x0fffffffull + ((ab >> 29) & 1ull)) >> 29) - (896ull << 23);
+  const float f = __uint_as_float((unsigned)rn | sign);
   float rf;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rf) : "f"(f));
-  double r = double(rf);
+  const unsigned rb = __float_as_uint(rf);
+  const uint64_t wide = ((uint64_t)(rb & 0x7fffffffu) << 29) + (896ull << 52) | ((uint64_t)(rb & 0x80000000u) << 32);
+  double r = __longlong_as_double((long long)wide);
   double e = fma(-d, r, 1.0);
   r = fma(r, e, r);
   e = fma(-d, r, 1.0);

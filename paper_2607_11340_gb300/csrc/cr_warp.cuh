@@ -42,6 +42,12 @@ CR_HD float recip_fast(float d) {
   return r;
 }
 CR_HD double recip_fast(double d) { return recip_nr(d); }
+// d > 0 (false for NaN); in FP64 on the bits, off the FP64 pipe (positive values are the bit patterns 1 .. that
+// of infinity).
+CR_HD bool positive(float d) { return d > 0.f; }
+CR_HD bool positive(double d) {
+  return (uint64_t)__double_as_longlong(d) - 1ull < 0x7ff0000000000000ull;
+}
 
 // Sweep of pivots 0..D-1 of the augmented matrix in the warp's slots. Pivot k maps d = S_kk to
 // -1/d, the rest of row and column k to S_ik / d and every other entry to S_ij - S_ik S_kj / d.
@@ -59,8 +65,9 @@ __device__ bool sweep_aug(V (&v)[AugSlots<D>::SL], const AugSlots<D>& sl, V* col
       if (sl.on[s] && (sl.r[s] == k || sl.c[s] == k)) col[sl.r[s] == k ? sl.c[s] : sl.r[s]] = v[s];
     __syncwarp();
     V d = col[k];
-    ok = ok && d > V(0);
-    d = d > V(0) ? d : V(1);
+    const bool pos = positive(d);
+    ok = ok && pos;
+    d = pos ? d : V(1);
     const V ri = recip_fast(d);
     if (lane <= D) colr[lane] = col[lane] * ri;
     __syncwarp();
