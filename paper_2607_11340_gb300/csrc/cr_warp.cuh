@@ -124,18 +124,28 @@ __device__ T warp_eval(const RobotK<T>& rb, const WeightsK<T>& w, const TargetK<
   // this lane's segment: twist (translational tv, angular tw for the two bending inputs), K, u
   T mtv[2][3], mtw[2][3], myK = T(0), myu = T(0), mysu = T(0);
   {
-    T tv[N][2][3], tw[N][2][3];
-    segment_twists(rb, ch, tv, tw);
+    // of this lane's segment only, as the last segment of a chain that ends there: a warp's chain of LM steps is
+    // bound by the latency of its instructions, and all N twists with a choice between them were 150 more per
+    // segment (512 paths x 64 waypoints, 4 segments: 32.3 -> 30.6 ms; 192 mixed items 103 -> 98 ms)
+    Chain<T, 1> own;
 #pragma unroll
     for (int ii = 0; ii < N; ++ii)
-      if (ii == myl) {
+      if (ii == 0 || ii == myl) {
 #pragma unroll
-        for (int k = 0; k < 2; ++k)
+        for (int a = 0; a < 9; ++a) own.Rb[0][a] = ch.Rb[ii][a];
 #pragma unroll
-          for (int a = 0; a < 3; ++a) { mtv[k][a] = tv[ii][k][a]; mtw[k][a] = tw[ii][k][a]; }
+        for (int a = 0; a < 3; ++a) own.p[a] = ii == N - 1 ? ch.p[a] : ch.pb[ii + 1 < N ? ii + 1 : ii][a];
+        own.ax[0] = ch.ax[ii]; own.ay[0] = ch.ay[ii]; own.x[0] = ch.x[ii];
+        own.s[0] = ch.s[ii]; own.c[0] = ch.c[ii]; own.L[0] = ch.L[ii];
         myK = rb.K[ii];
         mysu = u[3 * ii] + u[3 * ii + 1] + u[3 * ii + 2];
       }
+    T tv[1][2][3], tw[1][2][3];
+    segment_twists<T, 1>(rb, own, tv, tw);
+#pragma unroll
+    for (int k = 0; k < 2; ++k)
+#pragma unroll
+      for (int a = 0; a < 3; ++a) { mtv[k][a] = tv[0][k][a]; mtw[k][a] = tw[0][k][a]; }
 #pragma unroll
     for (int q = 0; q < D; ++q)
       if (q == lane) myu = u[q];
