@@ -1471,6 +1471,23 @@ template <> CR_HD void acc_prod<F2, float>(F2& acc, float x, float y) {
 CR_HD double to_f64(float v) { return double(v); }
 CR_HD double to_f64(double v) { return v; }
 CR_HD double to_f64(const F2& v) { return double(v.hi) + double(v.lo); }
+// The same without conversions, comparisons or maxima on the FP64 pipe, for kernels that it bounds (BITS): a
+// float as a double by shifting its bits (normal numbers and zeros; the rest by conversion), d > 0 and
+// max(d, lo) for lo > 0 by comparing bit patterns (false and lo for NaN).
+CR_HD double widen_bits(float v) {
+  const unsigned b = __float_as_uint(v), e = b & 0x7f800000u;
+  uint64_t w = ((uint64_t)(b & 0x7fffffffu) << 29) + (896ull << 52);
+  if (e == 0u || e == 0x7f800000u) {
+    if ((b << 1) != 0u) return double(v);
+    w = 0;
+  }
+  return __longlong_as_double((long long)(w | ((uint64_t)(b & 0x80000000u) << 32)));
+}
+CR_HD double to_f64_bits(const F2& v) { return widen_bits(v.hi) + widen_bits(v.lo); }
+CR_HD bool positive_bits(double d) { return (uint64_t)__double_as_longlong(d) - 1ull < 0x7ff0000000000000ull; }
+CR_HD double max_bits(double d, double lo) {
+  return positive_bits(d) && __double_as_longlong(d) > __double_as_longlong(lo) ? d : lo;
+}
 // The accumulator of an LM normal matrix for bulk precision T.
 template <typename T> struct NormalAcc { typedef T type; };
 template <> struct NormalAcc<float> { typedef F2 type; };
@@ -1827,7 +1844,7 @@ CR_HD double recip_nr(double d) {
 // Every loop has a constant trip count with the triangular range as a guard, so that full unrolling
 // leaves only constant indices and the packed matrix stays in registers (with trip counts that depend
 // on an outer index the compiler kept it in local memory).
-template <int D> CR_HD bool cholesky_packed(double (&A)[D * (D + 1) / 2], double (&invd)[D]) {
+template <int D, bool BITS = false> CR_HD bool cholesky_packed(double (&A)[D * (D + 1) / 2], double (&invd)[D]) {
   bool ok = true;  // no early exit: keeps the fully unrolled factorisation in registers
 #pragma unroll
   for (int j = 0; j < D; ++j) {
@@ -1835,8 +1852,14 @@ template <int D> CR_HD bool cholesky_packed(double (&A)[D * (D + 1) / 2], double
 #pragma unroll
     for (int k = 0; k < D; ++k)
       if (k < j) s -= A[tri(j, k)] * A[tri(j, k)];
-    ok = ok && (s > 0.0);
-    s = s > 0.0 ? s : 1.0;
+    if (BITS) {
+      const bool pos = positive_bits(s);
+      ok = ok && pos;
+      s = pos ? s : 1.0;
+    } else {
+      ok = ok && (s > 0.0);
+      s = s > 0.0 ? s : 1.0;
+    }
     double inv = rsqrt(s);
     double ljj = s * inv;
     invd[j] = inv;

@@ -64,7 +64,8 @@ CR_HD int pg_step(const RobotK<T>& rb, const WeightsK<T>& w, int kind, const Tar
 // ------------------------------------------------------------------------------------------------
 // One Levenberg-Marquardt iteration (Sec. IV-C); returns 1 if the step was accepted.
 // ------------------------------------------------------------------------------------------------
-template <typename T, int N, bool OBST, int MODEL = CR_MODEL_TENDON>
+// BITS (FP32): the FP64 part without conversions and comparisons on the FP64 pipe (to_f64_bits).
+template <typename T, int N, bool OBST, int MODEL = CR_MODEL_TENDON, bool BITS = false>
 CR_HD int lm_iteration(const RobotK<T>& rb, const WeightsK<T>& w, int kind, const TargetK<T>& tg,
                        ObsK<T> sph, int no, T (&u)[3 * N], double& lam, double& nu, T& Fout) {
   constexpr int D = 3 * N;
@@ -76,17 +77,24 @@ CR_HD int lm_iteration(const RobotK<T>& rb, const WeightsK<T>& w, int kind, cons
     typedef typename NormalAcc<T>::type TA;
     TA A[DD], g[D];
     F = eval_ik_normal<T, TA, N, OBST, MODEL>(rb, w, kind, tg, sph, no, u, A, g);
+    if constexpr (BITS) {
 #pragma unroll
-    for (int a = 0; a < DD; ++a) Ad[a] = to_f64(A[a]);
+      for (int a = 0; a < DD; ++a) Ad[a] = to_f64_bits(A[a]);
 #pragma unroll
-    for (int q = 0; q < D; ++q) dl[q] = to_f64(g[q]);
+      for (int q = 0; q < D; ++q) dl[q] = to_f64_bits(g[q]);
+    } else {
+#pragma unroll
+      for (int a = 0; a < DD; ++a) Ad[a] = to_f64(A[a]);
+#pragma unroll
+      for (int q = 0; q < D; ++q) dl[q] = to_f64(g[q]);
+    }
   }
 #pragma unroll
   for (int q = 0; q < D; ++q) {
-    Dg[q] = fmax(Ad[tri(q, q)], 1e-12);
+    Dg[q] = BITS ? max_bits(Ad[tri(q, q)], 1e-12) : fmax(Ad[tri(q, q)], 1e-12);
     Ad[tri(q, q)] += lam * Dg[q];
   }
-  if (!cholesky_packed<D>(Ad, invd)) {
+  if (!cholesky_packed<D, BITS>(Ad, invd)) {
     lam *= nu;
     nu *= 2.0;
     Fout = F;
@@ -465,7 +473,7 @@ CR_HD double accept_fp64(const RobotK<double>& rb, const WeightsK<double>& w, in
   return F;
 }
 
-template <typename T, int N, bool OBST, int MODEL = CR_MODEL_TENDON, bool PRIMS = true>
+template <typename T, int N, bool OBST, int MODEL = CR_MODEL_TENDON, bool PRIMS = true, bool BITS = false>
 __global__ void __launch_bounds__(128) k_ik_refine(RobotK<T> rb, WeightsK<T> w, RobotK<double> rbd,
                                                     WeightsK<double> wd, IkArgs<T> a) {
   constexpr int D = 3 * N;
@@ -506,7 +514,7 @@ __global__ void __launch_bounds__(128) k_ik_refine(RobotK<T> rb, WeightsK<T> w, 
     double lam = a.lambda0, nu = 2.0;
     T F;
     for (int it = 0; it < a.k_final; ++it)
-      lm_iteration<T, N, OBST, MODEL>(rb, w, a.kind, tg, sph, nob, u, lam, nu, F);
+      lm_iteration<T, N, OBST, MODEL, BITS>(rb, w, a.kind, tg, sph, nob, u, lam, nu, F);
   }
   double ud[D];
 #pragma unroll
@@ -938,7 +946,21 @@ template <typename T, int N, int MODEL = CR_MODEL_TENDON> cr_status solve_ik_n(c
       k_ik_refine<T, N, true, MODEL><<<g2, b2, sm2, a.stream>>>(rb, w, rbd, wd, k);
     }
   }
-  else k_ik_refine<T, N, false, MODEL><<<g2, b2, sm2, a.stream>>>(rb, w, rbd, wd, k);
+  else {
+    // Free space in FP32: with more than one warp to a sub-partition (4 x 152) the FP64 pipe sets the time and
+    // the form that keeps conversions and comparisons off it wins (3-segment IK of 4096 targets x 8 candidates
+    // 3.38 -> 3.23 ms in all); with fewer, a warp's own chain does, and the integer sequences are longer (100
+    // targets: 1.10 against 1.16 ms). Above 4 segments the state does not fit the registers and the form is
+    // slower at any size (5 segments, 3000 targets: 4.42 against 5.44 ms).
+    bool bits = false;
+    if constexpr (sizeof(T) == 4 && MODEL == CR_MODEL_TENDON && N <= 4) {
+      if (P * k.K > 32 * 4 * 152) {
+        k_ik_refine<T, N, false, MODEL, true, true><<<g2, b2, sm2, a.stream>>>(rb, w, rbd, wd, k);
+        bits = true;
+      }
+    }
+    if (!bits) k_ik_refine<T, N, false, MODEL><<<g2, b2, sm2, a.stream>>>(rb, w, rbd, wd, k);
+  }
   if ((st = crh::check_launch("cr_solve_ik refine"))) return st;
   k_ik_argmin<N><<<grid1(P, 128), 128, 0, a.stream>>>(P, k.K, k.pos_tol, k.rot_tol, k.cand_u64, k.cand_F,
                                                       k.cand_pos, k.cand_rot, k.cand_flag, k.u_out,
