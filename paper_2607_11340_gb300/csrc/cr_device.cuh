@@ -736,9 +736,7 @@ CR_HD void segment_sphere_masks(const RobotK<T>& rb, const Chain<T, N>& ch, ObsK
 // decides). One pass over the obstacles serves all segments: an obstacle's own part of the limit,
 // reach + 1e-4 (reach + |c|_1), is formed once, a test is then d^2 - lim^2 and its sign bit is shifted
 // into the mask (10 instructions a pair). Formed per segment with compares and 64-bit shifts a test took
-// about 20, half of the clearance work of a state among 64 spheres. Used where a decision or a cost of its own is
-// the result; the solvers' FP32 evaluations keep the form above, whose results ptxas rounds (fuses)
-// differently when the code beside them changes, which the projected-gradient iterates magnify.
+// about 20, half of the clearance work of a state among 64 spheres.
 template <int N>
 CR_HD void segment_sphere_masks_f(const Chain<float, N>& ch, ObsK<float> ob, int j0, int cnt, uint64_t (&mask)[N]) {
   const Sphere4<float>* sph = ob.s + j0;
@@ -774,6 +772,16 @@ CR_HD void segment_sphere_masks_f(const Chain<float, N>& ch, ObsK<float> ob, int
       mk = prim_exact_cull(ob, j0, mk, m[i][0], m[i][1], m[i][2], 0.5f * ch.L[i], lsum);
     mask[i] = mk;
   }
+}
+
+// The masks of the solvers' evaluations: FP32 takes the quicker form up to 4 segments (QUICK; 256 trajectories of
+// 32 states among 64 spheres 7.02 -> 6.56 ms, 512 paths 30.6 -> 30.0 ms). At 5 and 6 segments, and in the
+// trajectory solve of 4 among primitives, it gained as much, but with it beside them ptxas fuses the evaluation's
+// other sums differently, which the projected-gradient iterates magnify to other solutions; FP64 has no use for it.
+template <typename T, int N, bool QUICK = (N <= 4)>
+CR_HD void segment_masks(const RobotK<T>& rb, const Chain<T, N>& ch, ObsK<T> ob, int j0, int cnt, uint64_t (&mask)[N]) {
+  if constexpr (sizeof(T) == 4 && QUICK) segment_sphere_masks_f<N>(ch, ob, j0, cnt, mask);
+  else segment_sphere_masks(rb, ch, ob, j0, cnt, mask);
 }
 
 // Second level: the samples k0..k1 of segment i (arc fractions k / n_b) lie within
@@ -1071,9 +1079,9 @@ CR_HD void self_contact_forward(const RobotK<T>& rb, const WeightsK<T>& w, const
 // row would only add the rounding residue of the projection). OBST compiles the collision rows:
 // the spheres' and, with w.rho_s > 0, the self-contact rows (with_self = false leaves the latter to
 // another thread that evaluates the same state). FAST: the quicker search for near samples (CullView; in FP64
-// on the FP32 table f32), whose samples' rows are the same.
+// on the FP32 table f32), whose samples' rows are the same. QUICK: segment_masks' form.
 template <typename T, int N, bool OBST, bool GRAD, bool PGRAD, bool BOX = true, int MODEL = CR_MODEL_TENDON,
-          bool FAST = false>
+          bool FAST = false, bool QUICK = (N <= 4)>
 CR_HD T state_forward(const RobotK<T>& rb, const WeightsK<T>& w, ObsK<T> ob, int no,
                       const T (&u)[3 * N], Chain<T, N>& ch, StateAgg<T, N>& ag, T* coll_out,
                       bool with_self = true, const Sphere4<float>* f32 = nullptr) {
@@ -1098,7 +1106,7 @@ CR_HD T state_forward(const RobotK<T>& rb, const WeightsK<T>& w, ObsK<T> ob, int
 #pragma unroll
         for (int i = 0; i < N; ++i) smp[i] = mk[i] ? cv.samples(rb.nb, i, j0, mk[i]) : 0ull;
     } else {
-      segment_sphere_masks(rb, ch, ob, j0, no - j0 < 64 ? no - j0 : 64, mk);
+      segment_masks<T, N, QUICK>(rb, ch, ob, j0, no - j0 < 64 ? no - j0 : 64, mk);
     }
 #pragma unroll
     for (int i = 0; i < N; ++i) {
@@ -1675,7 +1683,7 @@ CR_HD T eval_ik_normal(const RobotK<T>& rb, const WeightsK<T>& w, int kind, cons
     const T inb = T(1) / T(rb.nb);
     for (int j0 = 0; j0 < no; j0 += 64) {
     uint64_t mk[N];
-    segment_sphere_masks(rb, ch, ob, j0, no - j0 < 64 ? no - j0 : 64, mk);
+    segment_masks(rb, ch, ob, j0, no - j0 < 64 ? no - j0 : 64, mk);
 #pragma unroll
     for (int i = 0; i < N; ++i) {
       if (!mk[i]) continue;
@@ -2072,7 +2080,7 @@ CR_HD bool state_collides(const RobotK<T>& rb, ObsK<T> ob, int no, const T (&u)[
   const T inb = T(1) / T(rb.nb);
   for (int j0 = 0; j0 < no; j0 += 64) {
     uint64_t mk[N];
-    segment_sphere_masks(rb, ch, ob, j0, no - j0 < 64 ? no - j0 : 64, mk);
+    segment_masks(rb, ch, ob, j0, no - j0 < 64 ? no - j0 : 64, mk);
     for (int i = 0; i < N; ++i) {
       if (!mk[i]) continue;
       for (int k0 = 1; k0 <= rb.nb; k0 += kCullGroup) {

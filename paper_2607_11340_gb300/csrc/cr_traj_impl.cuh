@@ -74,7 +74,7 @@ template <typename T> struct TrajSmem {
 // threads per state, each with its own part of the spheres (sph, no); the helper (aux = true) adds
 // only the clearance rows of its spheres to F and passes their force / moment aggregates to the
 // owner through shared memory, the owner runs everything else and hands the gradient back.
-template <typename T, int N, bool OBST, bool GRAD>
+template <typename T, int N, bool OBST, bool GRAD, bool QUICK = (N <= 4)>
 __device__ T traj_state_eval(const RobotK<T>& rb, const WeightsK<T>& w, const TrajW<T>& tw, int t, int Tn,
                              const T (&u)[3 * N], const TargetK<T>& goal, ObsK<T> sph, int no,
                              TrajSmem<T>& sm, T (&gu)[3 * N], bool split = false, bool aux = false) {
@@ -87,7 +87,8 @@ __device__ T traj_state_eval(const RobotK<T>& rb, const WeightsK<T>& w, const Tr
   if (aux) {
     if (active && t >= 1) {
       T coll = T(0);
-      state_forward<T, N, OBST, GRAD, false>(rb, w, sph, no, u, ch, ag, &coll, false);  // the owner has the self rows
+      state_forward<T, N, OBST, GRAD, false, true, CR_MODEL_TENDON, false, QUICK>(
+          rb, w, sph, no, u, ch, ag, &coll, false);  // the owner has the self rows
       F = coll;
       if (GRAD) {
         T* x = sm.xag + (size_t)t * 8 * N;
@@ -112,7 +113,7 @@ __device__ T traj_state_eval(const RobotK<T>& rb, const WeightsK<T>& w, const Tr
     if (t == 0) {
       chain_forward(rb, u, ch);  // the start state is fixed: only its tip enters the length rows
     } else {
-      F = state_forward<T, N, OBST, GRAD, false>(rb, w, sph, no, u, ch, ag, nullptr);
+      F = state_forward<T, N, OBST, GRAD, false, true, CR_MODEL_TENDON, false, QUICK>(rb, w, sph, no, u, ch, ag, nullptr);
     }
     if (t == Tn - 1) {
       T r[6], e[3], ang, sn, cs;
@@ -278,6 +279,7 @@ template <typename T, int N, bool OBST, bool PRIMS = true>
 __global__ void __launch_bounds__(256, 1) k_traj_solve(RobotK<T> rb, WeightsK<T> w, TrajW<T> tw, RobotK<double> rbd,
                                                      WeightsK<double> wd, TrajArgs<T> a) {
   constexpr int D = 3 * N;
+  constexpr bool QUICK = N <= 3 || (N == 4 && !PRIMS);  // see segment_masks
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int64_t p = blockIdx.x;
   const int Tn = a.Tn, Wt = ((Tn + 31) / 32) * 32;
@@ -313,7 +315,7 @@ __global__ void __launch_bounds__(256, 1) k_traj_solve(RobotK<T> rb, WeightsK<T>
   }
   TargetK<T> goal = load_target<T>(a.goal, a.P, p, CR_TASK_IK6);
   T g[D];
-  T F = block_sum(traj_state_eval<T, N, OBST, true>(rb, w, tw, t, Tn, u, goal, sph_m, no_m, sm, g, split, aux),
+  T F = block_sum(traj_state_eval<T, N, OBST, true, QUICK>(rb, w, tw, t, Tn, u, goal, sph_m, no_m, sm, g, split, aux),
                   sm.red);
   T alpha = a.alpha0;
   const bool free_state = active && t >= 1;
@@ -334,7 +336,7 @@ __global__ void __launch_bounds__(256, 1) k_traj_solve(RobotK<T> rb, WeightsK<T>
       }
     }
     T g1[D];
-    T F1 = block_sum(traj_state_eval<T, N, OBST, true>(rb, w, tw, t, Tn, u1, goal, sph_m, no_m, sm, g1, split, aux),
+    T F1 = block_sum(traj_state_eval<T, N, OBST, true, QUICK>(rb, w, tw, t, Tn, u1, goal, sph_m, no_m, sm, g1, split, aux),
                      sm.red);
     if (F1 < F) {
 #pragma unroll
