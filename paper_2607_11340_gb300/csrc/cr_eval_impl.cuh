@@ -5,6 +5,8 @@
 
 #include <cooperative_groups.h>
 
+#include <atomic>
+
 #include "cr_host.h"
 
 namespace crk {
@@ -160,13 +162,41 @@ __global__ void __launch_bounds__(kReduceThreads) k_reduce_rows(const T* __restr
   cl.sync();  // block 0 has read every block's sum before any of them exits
 }
 
+// Whether the current device can hold a cluster of 16 of these blocks, which is more than the 8 that every one
+// schedules: a partition of a GPU may not. Asked once per device and type, so that the order of the sums stays fixed.
+template <typename T> bool reduce_cluster16_fits() {
+  constexpr int kDevices = 64;
+  static std::atomic<int> known[kDevices];  // 0: not asked, 1: no, 2: yes
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kDevices) return false;
+  const int k = known[dev].load(std::memory_order_relaxed);
+  if (k) return k == 2;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(16, 1, 1);
+  cfg.blockDim = dim3(kReduceThreads, 1, 1);
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = 16;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  int clusters = 0;
+  const bool fits =
+      cudaFuncSetAttribute(k_reduce_rows<T>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+      cudaOccupancyMaxActiveClusters(&clusters, k_reduce_rows<T>, &cfg) == cudaSuccess && clusters > 0;
+  if (!fits) (void)cudaGetLastError();
+  known[dev].store(fits ? 2 : 1, std::memory_order_relaxed);
+  return fits;
+}
+
 // Blocks per row: enough for about one block per SM over all rows, a power of two of at most 16 (the
-// largest cluster, opt-in), and at least 2048 elements to a block, below which one block's few loads
-// cost less than the cluster's barriers.
-inline int reduce_cluster(int64_t rows, int64_t B) {
+// largest cluster, opt-in; 8 where that does not fit), and at least 2048 elements to a block, below which one
+// block's few loads cost less than the cluster's barriers.
+template <typename T> int reduce_cluster(int64_t rows, int64_t B) {
   int c = 1;
   while (c < 16 && rows * c < 152 && B >= (int64_t)4096 * c) c *= 2;
-  return c;
+  return c > 8 && !reduce_cluster16_fits<T>() ? 8 : c;
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -276,7 +306,7 @@ template <typename T> cr_status launch_cost_grad(const EvalArgs& a) {
 #define CR_EVAL_COUPLED_INSTANTIATE(EXT, T) EXT template void launch_eval_coupled<T>(const EvalArgs&, int);
 template <typename T>
 cr_status launch_reduce_rows(const void* x, int64_t rows, int64_t B, double* out, cudaStream_t s) {
-  const int c = reduce_cluster(rows, B);
+  const int c = reduce_cluster<T>(rows, B);
   for (int64_t r0 = 0; r0 < rows; r0 += 65535) {  // rows along grid.y
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)c, (unsigned)(rows - r0 < 65535 ? rows - r0 : 65535), 1);
