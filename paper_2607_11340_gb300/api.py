@@ -15,7 +15,7 @@ def robot_struct(spec: synth.RobotSpec) -> lib.cr_robot:
     n = spec.n
     r.n, r.m, r.n_b = n, 3, spec.nb
     r.model = lib.CR_MODEL_ARC if spec.is_arc else (lib.CR_MODEL_COUPLED if spec.coupled else lib.CR_MODEL_TENDON)
-    r.L[:n] = spec.L
+    r.L[:n] = list(spec.L)  # whatever indexes: tuple, list, array, tensor
     r.r_c[:n] = [spec.rc] * n
     r.u_max[:n] = [spec.umax] * n
     r.theta_max[:n] = [spec.thmax] * n
@@ -207,6 +207,11 @@ def solve_ik(robot_spec, ik_spec, weights, kind, targets_soa, scene=None, precis
 # ---------------------------------------------------------------------------------------------
 # Differentiation: the hand-written adjoint behind torch.autograd.Function (recompute-in-backward)
 # ---------------------------------------------------------------------------------------------
+def _numbers(v, n):
+    """v[0] .. v[n - 1] as floats: a row in one copy, other shapes (a column) entry by entry."""
+    return v.tolist()[:n] if v.ndim == 1 else [float(v[i]) for i in range(n)]
+
+
 class IkCost(torch.autograd.Function):
     """Per-state IK cost F_b(u_b; L, r_c). forward(u [d][B], L [n], r_c [n], ctx_data) -> cost [B].
 
@@ -220,8 +225,8 @@ class IkCost(torch.autograd.Function):
         spec, scene, task = ctx_data
         robot = robot_struct(spec)
         n = spec.n
-        robot.L[:n] = L.tolist()[:n]
-        robot.r_c[:n] = rc.tolist()[:n]
+        robot.L[:n] = _numbers(L, n)
+        robot.r_c[:n] = _numbers(rc, n)
         cost = torch.empty(u.shape[1], dtype=u.dtype, device=u.device)
         lib.cr_cost_grad(robot, scene.c, task, u.contiguous(), cost)
         ctx.save_for_backward(u)
