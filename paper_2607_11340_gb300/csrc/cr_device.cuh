@@ -829,8 +829,16 @@ template <typename T> CR_HD bool maybe_near(ObsK<T> ob, int j, const T (&x)[3], 
 
 // The quicker search for the near samples of one state (FAST). In FP64 it runs on an FP32 copy f of the obstacle
 // table and an FP32 chain of the same bends, down to the samples: it only has to leave a superset, and an FP64
-// instruction holds a sub-partition's unit 64 cycles. The FP32 backbone is within 2e-6 of the FP64 one relative to the
-// robot's length; the margins are 1e-4 (segments, groups) and 1e-5 (samples) of the magnitudes involved.
+// instruction holds a sub-partition's unit 64 cycles. The margins are 1e-4 (segments, groups) and 1e-5 (samples) of
+// the magnitudes involved. A bend of theta rad is off by at most 3e-7 theta in FP32 (five roundings) and turns what
+// follows it: with |bends| <= 16 over all segments that shifts a sample by up to 8e-6 of the robot's length, which with
+// 2e-6 for everything else stays within the samples' margin. Larger bends, robots whose size squared leaves FP32's
+// range, and tables with a sphere that does (f is null then) take every sample as near: the exact test of each pair
+// decides, as it does for the search's superset.
+constexpr float kCullMaxBend2 = 256.f, kCullMinLength = 1e-12f, kCullMaxLength = 1e15f, kCullMaxReach = 1e18f;
+// Whether the search may run on a table with an entry of this reach: the square of its limit is finite, and that of a
+// distance is finite or, where it overflows, not within the limit.
+CR_HD bool cull_entry_fits(float reach) { return reach <= kCullMaxReach; }
 template <typename T, int N> struct CullView {
   CR_HD CullView(const Chain<T, N>&, const Sphere4<float>*) {}
   CR_HD void masks(const Chain<T, N>& ch, ObsK<T> ob, int j0, int cnt, uint64_t (&mk)[N]) const {
@@ -842,12 +850,15 @@ template <int N> struct CullView<double, N> {
   Chain<float, N> cf;
   const Sphere4<float>* f;
   float slack;
+  bool all;  // every sample is taken as near
   CR_HD CullView(const Chain<double, N>& ch, const Sphere4<float>* f_) : f(f_), slack(0.f) {
+    float bend2 = 0.f;
     float R[9] = {1.f, 0.f, 0.f, 0.f, 1.f, 0.f, 0.f, 0.f, 1.f}, p[3] = {0.f, 0.f, 0.f};
 #pragma unroll
     for (int i = 0; i < N; ++i) {
       const float ax = float(ch.ax[i]), ay = float(ch.ay[i]), L = float(ch.L[i]), x = ax * ax + ay * ay;
       float s, c, Ri[9], di[3], t[3], Rn[9];
+      bend2 += x;
       seg_sc(x, s, c);
       seg_transform(ax, ay, x, s, c, L, Ri, di);
 #pragma unroll
@@ -866,13 +877,20 @@ template <int N> struct CullView<double, N> {
       for (int a = 0; a < 9; ++a) R[a] = Rn[a];
       slack = fmaf(1e-5f, L, slack);
     }
+    all = !(f && bend2 <= kCullMaxBend2 && slack >= 1e-5f * kCullMinLength && slack <= 1e-5f * kCullMaxLength);
   }
   CR_HD void masks(const Chain<double, N>&, ObsK<double>, int j0, int cnt, uint64_t (&mk)[N]) const {
+    if (all) {
+#pragma unroll
+      for (int i = 0; i < N; ++i) mk[i] = ~0ull >> (64 - cnt);
+      return;
+    }
     segment_sphere_masks_f<N>(cf, ObsK<float>(f), j0, cnt, mk);
   }
   // the samples of segment i (bit k - 1: sample k) that may be within reach of one of the candidates
   CR_HD uint64_t samples(int nb, int i, int j0, uint64_t cand) const {
     static_assert(CR_MAX_NB <= 64, "one bit per sample");
+    if (all) return ~0ull >> (64 - nb);
     const ObsK<float> of(f);
     const float inb = 1.f / float(nb);
     uint64_t smp = 0;

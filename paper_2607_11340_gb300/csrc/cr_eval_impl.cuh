@@ -79,10 +79,12 @@ __global__ void __launch_bounds__(128) k_cost_grad(RobotK<T> rb, WeightsK<T> w, 
     __syncthreads();
     if constexpr (sizeof(T) == 8) {  // the FP32 copy of the table for the broad phase
       Sphere4<float>* f = reinterpret_cast<Sphere4<float>*>(smem_raw + ((obstacles_smem<T>(no, np) + 15) & ~(size_t)15));
-      for (int j = threadIdx.x; j < no + np; j += blockDim.x)
+      bool fits = true;
+      for (int j = threadIdx.x; j < no + np; j += blockDim.x) {
         f[j] = Sphere4<float>{float(ob.s[j].x), float(ob.s[j].y), float(ob.s[j].z), float(ob.s[j].reach)};
-      f32 = f;
-      __syncthreads();
+        fits = fits && cull_entry_fits(f[j].reach);
+      }
+      f32 = __syncthreads_and(fits) ? f : nullptr;
     }
   }
   int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;

@@ -578,7 +578,9 @@ __global__ void __launch_bounds__(256, 1) k_ik_refine_warp(RobotK<float> rb, Wei
       for (int q = 0; q < D; ++q) sud[wid * D + q] = double(u[q]);
     }
   }
-  __syncthreads();
+  bool fits = true;
+  for (int j = threadIdx.x; j < nob; j += blockDim.x) fits = fits && cull_entry_fits(sph.s[j].reach);
+  fits = __syncthreads_and(fits);
   // FP64 acceptance, one lane per candidate (the FP64 pipe charges whole warps: K lanes of one warp
   // instead of K warps running the same check in all their lanes)
   if (wid == 0 && lane < a.K) {
@@ -591,7 +593,7 @@ __global__ void __launch_bounds__(256, 1) k_ik_refine_warp(RobotK<float> rb, Wei
     if (isfinite(ud[0])) {
       const TargetK<double> tgd = load_target<double>(a.targets, a.P, p, CR_TASK_IK6);
       F = accept_fp64<N, true, CR_MODEL_TENDON, true>(rbd, wd, CR_TASK_IK6, tgd, sphd, nob, ud, a.lim_tol, pos, rot, flags,
-                                                      sph.s);
+                                                      fits ? sph.s : nullptr);
     }
 #pragma unroll
     for (int q = 0; q < D; ++q) a.cand_u64[q * PK + c] = ud[q];
