@@ -132,7 +132,7 @@ cr_status check_items(const cr_robot* family, const cr_batch_item* items, int64_
 
 // Host-side plan of one batch: per-item offsets, the queues per segment count and the workspace
 // layout. Estimated costs (relative warp time) order the queues longest first. grid[n-1]: the four
-// phase kernels' grids; the joint phase's warps get the per-worker path buffers.
+// phase kernels' grids; the joint phase's workers (warps, or blocks in its block form) get a set of path buffers each.
 struct Layout {
   std::vector<crk::BatchItemK> items;  // grouped by n, queue order inside a group
   std::vector<int2> units;             // grouped by n
@@ -225,8 +225,9 @@ cr_status make_layout(const cr_batch_item* items, int64_t N, const cr_batch_para
         L.grid[n - 1].g[ph] = (int)((work[ph] + wpb - 1) / wpb);
       }
     }
-    // joint phase of few path items: a block to an item, as long as all of them are resident at once (two
-    // blocks of 255 registers a thread to an SM); more items keep the chip busy with a warp to each
+    // joint phase of few path items: a block to an item, as long as this segment count's would all be resident at
+    // once on an idle device (two blocks of 255 registers a thread to an SM; the branches of the other segment counts
+    // share it); more items keep the chip busy with a warp to each
     L.grid[n - 1].joint_blocks = npath > 0 && npath <= 2 * (int64_t)n_sm ? (int)npath : 0;
     L.workers += (int64_t)L.grid[n - 1].g[0] * crk::kBatchWarps;
   }

@@ -14,10 +14,11 @@
 //  k_batch_warm:   per path item, the exploration sweep (warm-started LM per waypoint) into the
 //                  buffer;
 //  k_batch_joint:  per path item, the joint LM over the waypoints, the FP64 acceptance of every
-//                  waypoint and the outputs.
-// No warp waits for another. The segment counts run as parallel branches, behind a node that
-// zeroes the queue heads and stamps the batch start (%globaltimer); every item records its
-// completion time.
+//                  waypoint and the outputs; k_batch_joint_block does the same with a block of four warps
+//                  to an item where the path items of a segment count are few.
+// No warp waits for another, but for the four of a k_batch_joint_block block at its barriers. The segment
+// counts run as parallel branches, behind a node that zeroes the queue heads and stamps the batch start
+// (%globaltimer); every item records its completion time.
 #pragma once
 
 #include "cr_path_impl.cuh"
@@ -46,7 +47,7 @@ struct BatchArgs {
   int64_t W;
   const double* spheres;    // [*][4]
   float* cand;
-  unsigned char* scratch;   // per worker warp of the joint phase: path buffers
+  unsigned char* scratch;   // path buffers of the joint phase, one set per worker (a warp, or a block of the block form)
   size_t scratch_stride;
   int32_t hmax;             // waypoints the path buffers hold
   int32_t spu;              // seeds per unit
@@ -66,7 +67,7 @@ struct BatchArgs {
   unsigned long long* t_done;
 };
 
-constexpr int kBatchWarps = 4;         // warps per CTA (independent workers)
+constexpr int kBatchWarps = 4;         // warps per CTA (independent workers but in the joint phase's block form)
 constexpr int kBatchMaxSpheres = 64;   // obstacles per item
 constexpr size_t kBatchWarpSmem = 6144;
 
@@ -654,7 +655,7 @@ __device__ double joint_lm_block(const RobotK<float>& rb, const WeightsK<float>&
 }
 
 // Phase 4 with a block to a path item, for batches whose path items of one segment count are few (see
-// batch_joint_blocks): one warp's share of a long path, 128 waypoints in four rounds of evaluations, sets the
+// joint_blocks in make_layout): one warp's share of a long path, 128 waypoints in four rounds of evaluations, sets the
 // time of such a batch (63 of 116 ms for 192 mixed items, 6 segments).
 template <int N>
 __global__ void __maxnreg__(255)

@@ -462,10 +462,6 @@ CR_HD void seg_coef_poly(double x, double& s, double& c, double& s3, double& cp)
     seg_deriv_lib(x, s, c, s3, cp);
   }
 }
-template <typename T, int N>
-__device__ void calib_pose(const RobotK<T>& rb, const T (&u)[3 * N], const double* pm, T (&r)[3], T (&J)[3][2 * N]) {
-  calib_rows<T, N>(rb, u, pm, r, J);
-}
 template <int N>
 __device__ void calib_pose_f64(const RobotK<double>& rb, const double (&u)[3 * N], const double* pm, double (&r)[3],
                                double (&J)[3][2 * N]) {
@@ -537,7 +533,7 @@ __device__ void calib_pose_f64(const RobotK<double>& rb, const double (&u)[3 * N
 // evaluation (its cost is F). All sums have a fixed order: a lane adds one entry over its warp's poses in
 // order, the block its warps, every block the blocks' partials in four runs; F adds tile totals t, t + 32,
 // ... on lane t and then the lanes, which the single-block cost kernel repeats.
-// Bound: the FP64 pipe and its latency; 1024 poses are 32 warps on 32 of 608 sub-partitions, each busy with
+// Bound: the FP64 pipe and its latency; 1024 poses are 32 warps in 8 blocks, on 32 of 608 sub-partitions, each busy with
 // its own poses' instructions. 20 iterations of 1024 poses in FP64: 0.50 ms; as two launches an iteration, the
 // second one block that evaluated the trial cost of all poses on one SM, 2.57 ms.
 constexpr int kCalibThreads = 128, kCalibWarps = kCalibThreads / 32;
@@ -583,7 +579,7 @@ __device__ void calib_load_pose(const RobotK<T>& rb, const T* __restrict__ U, co
   for (int q = 0; q < D; ++q) u[q] = U[q * K + k];
   const double pm[3] = {Pm[k], Pm[K + k], Pm[2 * K + k]};
   if constexpr (sizeof(T) == 8) calib_pose_f64<N>(rb, u, pm, r, J);
-  else calib_pose<T, N>(rb, u, pm, r, J);
+  else calib_rows<T, N>(rb, u, pm, r, J);
 }
 // 1/2 |r|^2 of a tile, the same in every lane.
 template <typename T> __device__ double calib_tile_cost(const T (&r)[3]) {

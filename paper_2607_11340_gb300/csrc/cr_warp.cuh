@@ -42,12 +42,9 @@ CR_HD float recip_fast(float d) {
   return r;
 }
 CR_HD double recip_fast(double d) { return recip_nr(d); }
-// d > 0 (false for NaN); in FP64 on the bits, off the FP64 pipe (positive values are the bit patterns 1 .. that
-// of infinity).
+// d > 0 (false for NaN); in FP64 on the bits, off the FP64 pipe.
 CR_HD bool positive(float d) { return d > 0.f; }
-CR_HD bool positive(double d) {
-  return (uint64_t)__double_as_longlong(d) - 1ull < 0x7ff0000000000000ull;
-}
+CR_HD bool positive(double d) { return positive_bits(d); }
 
 // Sweep of pivots 0..D-1 of the augmented matrix in the warp's slots. Pivot k maps d = S_kk to
 // -1/d, the rest of row and column k to S_ik / d and every other entry to S_ij - S_ik S_kj / d.
@@ -321,12 +318,13 @@ template <typename T, int D> struct WarpNormal {
   bool solved;  // the scratch sdg holds this A's damping diagonal
 };
 
-// Relative half spacing of T's numbers below a power of two: |d| < |u| tiny_step gives u + d == u.
+// |d| < |u| tiny_step gives u + d == u: T's numbers below |u| are at least |u| 2^-24 (2^-53) apart, half of that is the
+// bound of rounding back to u, and this is half of it again.
 template <typename T> CR_HD constexpr T tiny_step() { return sizeof(T) == 4 ? T(1.0 / 67108864.0) : T(1.0 / 36028797018963968.0); }
 
 // Whether every further iteration is a rejection that leaves u: the step is delta = -(A + lambda D)^-1 g,
 // so with A >= 0 (up to rounding, which lambda >= 1 covers) |delta_q| sqrt(D_q) <= |D^-1/2 g| / lambda.
-// Where twice that bound is below the spacing of u_q for every q, u + delta rounds to u, the trial is
+// Where twice that bound is below |u_q| tiny_step for every q, u + delta rounds to u, the trial is
 // the state itself, its cost is F, and lambda only grows. Evaluated by the whole warp; sdg holds D.
 template <typename T, int D, typename V>
 __device__ bool warp_frozen(const T (&u)[D], T gq, const V* sdg, V lam) {
