@@ -120,10 +120,11 @@ __global__ void __launch_bounds__(128) k_cost_grad(RobotK<T> rb, WeightsK<T> w, 
 // 64 cycles). One block of 256 threads with one load in flight per row kept 6 SMs busy on the 6
 // parameter rows of 262,144 states and waited on every load: 195 us of a 485 us gradient pass, which takes
 // 328 us with 16 blocks per row (60,001 states and 8 rows: 52 us of 396, now 359).
-constexpr int kReduceThreads = 512, kReduceWarps = kReduceThreads / 32;
-template <typename T>
-__global__ void __launch_bounds__(kReduceThreads) k_reduce_rows(const T* __restrict__ x, int64_t B, double* out) {
-  __shared__ double part[kReduceWarps];
+constexpr int kReduceThreads = 512;  // of a cluster's blocks
+template <typename T, int TH>
+__global__ void __launch_bounds__(TH) k_reduce_rows(const T* __restrict__ x, int64_t B, double* out) {
+  constexpr int NW = TH / 32;
+  __shared__ double part[NW];
   __shared__ double total;
   namespace cg = cooperative_groups;
   const int64_t len = (B + gridDim.x - 1) / gridDim.x;
@@ -131,22 +132,35 @@ __global__ void __launch_bounds__(kReduceThreads) k_reduce_rows(const T* __restr
   const T* row = x + (int64_t)blockIdx.y * B;
   double acc[4] = {0.0, 0.0, 0.0, 0.0};
   int64_t b = b0 + threadIdx.x;
-  for (; b + 7 * kReduceThreads < b1; b += 8 * kReduceThreads) {
+  for (; b + 7 * TH < b1; b += 8 * TH) {
     T v[8];
 #pragma unroll
-    for (int k = 0; k < 8; ++k) v[k] = row[b + k * kReduceThreads];
+    for (int k = 0; k < 8; ++k) v[k] = row[b + k * TH];
 #pragma unroll
     for (int k = 0; k < 8; ++k) acc[k & 3] += double(v[k]);
   }
-  for (; b < b1; b += kReduceThreads) acc[0] += double(row[b]);
+  if (NW == 1) {  // the last elements: in flight together where no other warp hides their latency
+    T v[7];
+#pragma unroll
+    for (int k = 0; k < 7; ++k) v[k] = b + k * TH < b1 ? row[b + k * TH] : T(0);
+#pragma unroll
+    for (int k = 0; k < 7; ++k)
+      if (b + k * TH < b1) acc[0] += double(v[k]);
+  } else {
+    for (; b < b1; b += TH) acc[0] += double(row[b]);
+  }
   double s = (acc[0] + acc[1]) + (acc[2] + acc[3]);
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
-  if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = s;
-  __syncthreads();
+  if (NW > 1) {
+    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = s;
+    __syncthreads();
+  }
   if (threadIdx.x == 0) {
-    s = part[0];
-    for (int w = 1; w < kReduceWarps; ++w) s += part[w];
+    if (NW > 1) {
+      s = part[0];
+      for (int w = 1; w < NW; ++w) s += part[w];
+    }
     total = s;
   }
   if (gridDim.x == 1) {
@@ -185,8 +199,9 @@ template <typename T> bool reduce_cluster16_fits() {
   cfg.numAttrs = 1;
   int clusters = 0;
   const bool fits =
-      cudaFuncSetAttribute(k_reduce_rows<T>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
-      cudaOccupancyMaxActiveClusters(&clusters, k_reduce_rows<T>, &cfg) == cudaSuccess && clusters > 0;
+      cudaFuncSetAttribute(k_reduce_rows<T, kReduceThreads>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) ==
+          cudaSuccess &&
+      cudaOccupancyMaxActiveClusters(&clusters, k_reduce_rows<T, kReduceThreads>, &cfg) == cudaSuccess && clusters > 0;
   if (!fits) (void)cudaGetLastError();
   known[dev].store(fits ? 2 : 1, std::memory_order_relaxed);
   return fits;
@@ -199,6 +214,18 @@ template <typename T> int reduce_cluster(int64_t rows, int64_t B) {
   int c = 1;
   while (c < 16 && rows * c < 152 && B >= (int64_t)4096 * c) c *= 2;
   return c > 8 && !reduce_cluster16_fits<T>() ? 8 : c;
+}
+
+// Threads of a block: 512 in a cluster. A row that is one block's (many rows, or short ones) takes fewer: every warp
+// adds 8 FP64 operations of its own, which bound short rows (100,000 rows of 300 in FP32: 1.45 ms with 512 threads, 0.52
+// with 128, 0.23 with a warp). With a warp or more to each of the 4 x 152 sub-partitions a row of up to 8192
+// elements is one warp's (1000 rows of 1000: 10 us, 25 with 512 threads); fewer rows have 128 threads (304 rows of 4096: 8
+// us, 14 with a warp), and above 16,384 elements 256 keep more loads in flight (1000 rows of 30,000 in FP64: 72 us, 77
+// with 128, 80 with 512).
+inline int reduce_threads(int c, int64_t rows, int64_t B) {
+  if (c > 1) return kReduceThreads;
+  if (rows >= 608 && B <= 8192) return 32;
+  return B <= 16384 ? 128 : 256;
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -309,10 +336,13 @@ template <typename T> cr_status launch_cost_grad(const EvalArgs& a) {
 template <typename T>
 cr_status launch_reduce_rows(const void* x, int64_t rows, int64_t B, double* out, cudaStream_t s) {
   const int c = reduce_cluster<T>(rows, B);
+  const int th = reduce_threads(c, rows, B);
+  auto kernel = th == 32 ? k_reduce_rows<T, 32> : th == 128 ? k_reduce_rows<T, 128>
+              : th == 256 ? k_reduce_rows<T, 256> : k_reduce_rows<T, kReduceThreads>;
   for (int64_t r0 = 0; r0 < rows; r0 += 65535) {  // rows along grid.y
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)c, (unsigned)(rows - r0 < 65535 ? rows - r0 : 65535), 1);
-    cfg.blockDim = dim3(kReduceThreads, 1, 1);
+    cfg.blockDim = dim3((unsigned)th, 1, 1);
     cfg.stream = s;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
@@ -322,8 +352,8 @@ cr_status launch_reduce_rows(const void* x, int64_t rows, int64_t B, double* out
     cfg.attrs = at;
     cfg.numAttrs = c > 1 ? 1 : 0;
     cudaError_t e = cudaSuccess;
-    if (c > 8) e = cudaFuncSetAttribute(k_reduce_rows<T>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    if (e == cudaSuccess) e = cudaLaunchKernelEx(&cfg, k_reduce_rows<T>, (const T*)x + r0 * B, B, out + r0);
+    if (c > 8) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e == cudaSuccess) e = cudaLaunchKernelEx(&cfg, kernel, (const T*)x + r0 * B, B, out + r0);
     if (e != cudaSuccess) {
       (void)cudaGetLastError();
       return crh::fail(CR_ECUDA, "cr_reduce_rows: %s", cudaGetErrorString(e));
