@@ -879,13 +879,24 @@ template <int N> struct CullView<double, N> {
     }
     all = !(f && bend2 <= kCullMaxBend2 && slack >= 1e-5f * kCullMinLength && slack <= 1e-5f * kCullMaxLength);
   }
-  CR_HD void masks(const Chain<double, N>&, ObsK<double>, int j0, int cnt, uint64_t (&mk)[N]) const {
+  CR_HD void masks(const Chain<double, N>&, ObsK<double> ob, int j0, int cnt, uint64_t (&mk)[N]) const {
     if (all) {
 #pragma unroll
       for (int i = 0; i < N; ++i) mk[i] = ~0ull >> (64 - cnt);
       return;
     }
     segment_sphere_masks_f<N>(cf, ObsK<float>(f), j0, cnt, mk);
+    if (!ob.prims()) return;
+    // f has the primitives' bounding spheres only: those candidates are culled by the signed distance as without FAST
+    const uint64_t sb = sphere_bits(ob, j0);
+#pragma unroll
+    for (int i = 0; i < N; ++i)
+      if (mk[i] & ~sb) {
+        float q[3], m[3], s, c;
+        backbone_point(cf.Rb[i], cf.pb[i], cf.ax[i], cf.ay[i], cf.x[i], cf.L[i], 0.5f, q, m, s, c);
+        mk[i] = prim_exact_cull(ob, j0, mk[i], double(m[0]), double(m[1]), double(m[2]), 0.5 * double(cf.L[i]),
+                                1e5 * double(slack));
+      }
   }
   // the samples of segment i (bit k - 1: sample k) that may be within reach of one of the candidates
   CR_HD uint64_t samples(int nb, int i, int j0, uint64_t cand) const {
@@ -1132,7 +1143,15 @@ CR_HD T state_forward(const RobotK<T>& rb, const WeightsK<T>& w, ObsK<T> ob, int
       constexpr bool picked = FAST && sizeof(T) == 8;
       for (int k0 = 1; k0 <= rb.nb; k0 += kCullGroup) {
       const int k1 = k0 + kCullGroup - 1 < rb.nb ? k0 + kCullGroup - 1 : rb.nb;
-      const uint64_t gm = picked ? mk[i] : group_sphere_mask<T, N>(rb.nb, ch, i, k0, k1, ob, j0, mk[i]);
+      uint64_t gm;
+      if constexpr (picked) {
+        if (!((smp[i] >> (k0 - 1)) & ((1ull << kCullGroup) - 1ull))) continue;
+        gm = mk[i];
+        const uint64_t pm = ob.prims() ? gm & ~sphere_bits(ob, j0) : 0ull;  // a primitive's test is the dear one
+        if (pm) gm = (gm & ~pm) | group_sphere_mask<T, N>(rb.nb, ch, i, k0, k1, ob, j0, pm);
+      } else {
+        gm = group_sphere_mask<T, N>(rb.nb, ch, i, k0, k1, ob, j0, mk[i]);
+      }
       if (!gm) continue;
       for (int k = k0; k <= k1; ++k) {
         if (picked && !((smp[i] >> (k - 1)) & 1ull)) continue;
