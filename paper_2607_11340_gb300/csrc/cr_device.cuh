@@ -736,7 +736,9 @@ CR_HD void segment_sphere_masks(const RobotK<T>& rb, const Chain<T, N>& ch, ObsK
 // decides). One pass over the obstacles serves all segments: an obstacle's own part of the limit,
 // reach + 1e-4 (reach + |c|_1), is formed once, a test is then d^2 - lim^2 and its sign bit is shifted
 // into the mask (10 instructions a pair). Formed per segment with compares and 64-bit shifts a test took
-// about 20, half of the clearance work of a state among 64 spheres.
+// about 20, half of the clearance work of a state among 64 spheres. With one segment there is nothing to share: 4
+// tests side by side, as the former loop had them (trajectory cost among 200 spheres 18.7 us, 20.6 one by one, now
+// 16.5); with more segments their tests already are, and longer loops only cost fetches.
 template <int N>
 CR_HD void segment_sphere_masks_f(const Chain<float, N>& ch, ObsK<float> ob, int j0, int cnt, uint64_t (&mask)[N]) {
   const Sphere4<float>* sph = ob.s + j0;
@@ -761,9 +763,9 @@ CR_HD void segment_sphere_masks_f(const Chain<float, N>& ch, ObsK<float> ob, int
       w[i] = __funnelshift_l(__float_as_uint(v), w[i], 1);  // (w << 1) | sign of v
     }
   };
-#pragma unroll 1
+#pragma unroll(N == 1 ? 4 : 1)
   for (int j = cnt - 1; j >= 32; --j) test(j, hi);
-#pragma unroll 2
+#pragma unroll(N == 1 ? 4 : 2)
   for (int j = (cnt < 32 ? cnt : 32) - 1; j >= 0; --j) test(j, lo);
 #pragma unroll
   for (int i = 0; i < N; ++i) {
