@@ -952,11 +952,13 @@ template <typename T, int N, int MODEL = CR_MODEL_TENDON> cr_status solve_ik_n(c
     // Free space in FP32: with more than one warp to a sub-partition (4 x 152) the FP64 pipe sets the time and
     // the form that keeps conversions and comparisons off it wins (3-segment IK of 4096 targets x 8 candidates
     // 3.38 -> 3.23 ms in all); with fewer, a warp's own chain does, and the integer sequences are longer (100
-    // targets: 1.10 against 1.16 ms). Above 4 segments the state does not fit the registers and the form is
-    // slower at any size (5 segments, 3000 targets: 4.42 against 5.44 ms).
+    // targets: 1.10 against 1.16 ms). With 3 segments that holds up to one and a half (the refine alone: 21,000
+    // candidates 1.03 against 1.13 ms, 29,000 1.19 against 1.18, 31,000 1.37 against 1.20); with 4 the two are equal
+    // from one on (19,500 candidates 1.84 ms, 31,000 2.46 against 2.03). Above 4 segments the state does not fit the
+    // registers and the form is slower at any size (5 segments, 3000 targets: 4.42 against 5.44 ms).
     bool bits = false;
     if constexpr (sizeof(T) == 4 && MODEL == CR_MODEL_TENDON && N <= 4) {
-      if (P * k.K > 32 * 4 * 152) {
+      if (P * k.K > (N == 3 ? 48 : 32) * 4 * 152) {
         k_ik_refine<T, N, false, MODEL, true, true><<<g2, b2, sm2, a.stream>>>(rb, w, rbd, wd, k);
         bits = true;
       }
