@@ -227,7 +227,8 @@ CR_API cr_status cr_cost_grad(const cr_robot* robot, const cr_scene* scene, cons
                        void* grad_param_out, int32_t dtype, cr_stream stream);
 
 /* Deterministic row sums: out[r] = sum_b x[r][b] for r < rows (x [rows][B] in `dtype`, out FP64).
- * One block per row, fixed summation order (used to reduce per-state parameter gradients). */
+ * A row is added by a warp, a block or a cluster of up to 16 blocks, by its length, the number of rows and
+ * what the device can hold; the order is fixed by these (used to reduce per-state parameter gradients). */
 CR_API cr_status cr_reduce_rows(const void* x, int64_t rows, int64_t B, double* out, int32_t dtype,
                          cr_stream stream);
 
